@@ -72,6 +72,14 @@ __device__ __forceinline__ bool checked(bool ok, int* err) {
   }
 }
 
+// Step constants of a lattice in a kernel's arithmetic type.
+template <typename T>
+struct LatConst {
+  T sigma, beta, s_e, s_eps, s_q, rho0, u_in, rho_out, grad_eps;
+  T h_inv_nuR, h_inv_nuB;   // 1/(2 nu_R), 1/(2 nu_B): the two weights of Eq. 18
+  T cos_theta;              // cos(theta) of the surface-energy variant
+};
+
 // Per-lattice constants, resident in global memory, one entry per lattice of a handle.
 struct LatDev {
   int nx, ny, pitch, bcx, bcy, in_prof;   // in_prof: 1 = Poiseuille inlet profile
@@ -83,6 +91,15 @@ struct LatDev {
   double in_y0, in_w;           // inlet profile: s = (y - in_y0) / in_w across the channel
   int wetting, pad2_;           // 0: improved scheme (a); 1: scheme (b), Eq. 48; 2: surface energy
   double cos_theta;             // cos(theta) of the surface-energy variant
+  // the same constants rounded to FP32 on the host: a kernel that computes in FP32 otherwise
+  // converts about ten doubles per thread, on an FP64 pipe of two lanes per SM
+  LatConst<float> cf;
+  template <typename T>
+  __host__ __device__ LatConst<T> consts() const {
+    if constexpr (sizeof(T) == 4) return cf;
+    else return LatConst<T>{T(sigma),   T(beta),     T(s_e),       T(s_eps),     T(s_q),        T(rho0), T(u_in),
+                            T(rho_out), T(grad_eps), T(h_inv_nuR), T(h_inv_nuB), T(cos_theta)};
+  }
 };
 
 // Inlet velocity of row y (Sec. III.D): uniform u_in, or the Poiseuille profile
@@ -108,6 +125,23 @@ template <typename T>
 __host__ __device__ constexpr T wgt(int a) {
   return a == 0 ? T(4.0 / 9.0) : (a <= 4 ? T(1.0 / 9.0) : T(1.0 / 36.0));
 }
+
+// ------------------------------------------------------------------ rounding-exact helpers
+// The wall chain (Eq. 28-36) is evaluated without contraction into fused multiply-adds and
+// in a fixed order, so that exact cancellations (e.g. a gradient exactly normal to a flat
+// wall, which makes D1 == D2 in Eq. 35-36 an exact tie) are reproduced exactly.
+__device__ __forceinline__ double radd(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double rsub(double a, double b) { return __dsub_rn(a, b); }
+__device__ __forceinline__ double rmul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double rdiv(double a, double b) { return __ddiv_rn(a, b); }
+__device__ __forceinline__ double rsqrt_(double a) { return __dsqrt_rn(a); }
+__device__ __forceinline__ float radd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float rsub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float rmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float rdiv(float a, float b) { return __fdiv_rn(a, b); }
+__device__ __forceinline__ float rsqrt_(float a) { return __fsqrt_rn(a); }
+__device__ __forceinline__ double fma_(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float fma_(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 
 // ------------------------------------------------------------------ storage traits
 template <typename S> struct Store;
@@ -165,8 +199,8 @@ __device__ __forceinline__ uint32_t cvt_rs_bf16x2(float lo, float hi, uint32_t r
 }
 // key of one step of one lattice: epoch counts graph replays (device counter), step the
 // launch within them (or the absolute step of a direct launch)
-__device__ __forceinline__ uint32_t sr_key(const uint32_t* epoch, uint32_t step, long long pop_off) {
-  return hash32(hash32(*epoch ^ 0x9E3779B9u) + step) + uint32_t(pop_off);
+__device__ __forceinline__ uint32_t sr_key(uint32_t epoch, uint32_t step, long long pop_off) {
+  return hash32(hash32(epoch ^ 0x9E3779B9u) + step) + uint32_t(pop_off);
 }
 
 // FP16 keeps d and g scaled by 2^10: an exact power of two that leaves the rounding of
@@ -246,28 +280,13 @@ __device__ __forceinline__ void decode(T lo, T hi, T wr0, T& fr, T& fb) {
 template <typename S, typename T>
 __device__ __forceinline__ void encode(T fr, T fb, T wr0, T& lo, T& hi) {
   if constexpr (Store<S>::kDeviation) {
-    lo = ((fr + fb) - wr0) * Store<S>::kScale;
-    hi = (fr - fb) * Store<S>::kScale;
+    lo = rmul(rsub(radd(fr, fb), wr0), Store<S>::kScale);
+    hi = rmul(rsub(fr, fb), Store<S>::kScale);
   } else {
     lo = fr;
     hi = fb;
   }
 }
-
-// ------------------------------------------------------------------ rounding-exact helpers
-// The wall chain (Eq. 28-36) is evaluated without contraction into fused multiply-adds and
-// in a fixed order, so that exact cancellations (e.g. a gradient exactly normal to a flat
-// wall, which makes D1 == D2 in Eq. 35-36 an exact tie) are reproduced exactly.
-__device__ __forceinline__ double radd(double a, double b) { return __dadd_rn(a, b); }
-__device__ __forceinline__ double rsub(double a, double b) { return __dsub_rn(a, b); }
-__device__ __forceinline__ double rmul(double a, double b) { return __dmul_rn(a, b); }
-__device__ __forceinline__ double rdiv(double a, double b) { return __ddiv_rn(a, b); }
-__device__ __forceinline__ double rsqrt_(double a) { return __dsqrt_rn(a); }
-__device__ __forceinline__ float radd(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ float rsub(float a, float b) { return __fsub_rn(a, b); }
-__device__ __forceinline__ float rmul(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ float rdiv(float a, float b) { return __fdiv_rn(a, b); }
-__device__ __forceinline__ float rsqrt_(float a) { return __fsqrt_rn(a); }
 
 // ------------------------------------------------------------------ neighbour mapping
 // Periodic axes wrap; other axes clamp (on an inlet/outlet axis the clamped ghost column
@@ -299,10 +318,11 @@ __device__ __forceinline__ void zou_he(int x, int nx, T u_in, T rho_out, T fr[9]
 #pragma unroll
     for (int a = 0; a < 9; ++a) f[a] = fr[a] + fb[a];
     const T u = u_in;
-    const T rho = zh_div(f[0] + f[2] + f[4] + T(2) * (f[3] + f[6] + f[7]), T(1) - u);
-    f[1] = f[3] + T(2.0 / 3.0) * rho * u;
-    f[5] = f[7] - T(0.5) * (f[2] - f[4]) + rho * u / T(6);
-    f[8] = f[6] + T(0.5) * (f[2] - f[4]) + rho * u / T(6);
+    const T rho = zh_div(fma_(T(2), radd(radd(f[3], f[6]), f[7]), radd(radd(f[0], f[2]), f[4])), rsub(T(1), u));
+    const T d = rsub(f[2], f[4]), q = rdiv(rmul(rho, u), T(6));
+    f[1] = fma_(rmul(T(2.0 / 3.0), rho), u, f[3]);
+    f[5] = radd(fma_(T(-0.5), d, f[7]), q);
+    f[8] = radd(fma_(T(0.5), d, f[6]), q);
 #pragma unroll
     for (int a = 0; a < 9; ++a) {
       fr[a] = f[a];
@@ -313,19 +333,21 @@ __device__ __forceinline__ void zou_he(int x, int nx, T u_in, T rho_out, T fr[9]
 #pragma unroll
     for (int a = 0; a < 9; ++a) f[a] = fr[a] + fb[a];
     const T r = rho_out;
-    const T ux = T(-1) + zh_div(f[0] + f[2] + f[4] + T(2) * (f[1] + f[5] + f[8]), r);
-    const T f3 = f[1] - T(2.0 / 3.0) * r * ux;
-    const T f7 = f[5] + T(0.5) * (f[2] - f[4]) - r * ux / T(6);
-    const T f6 = f[8] - T(0.5) * (f[2] - f[4]) - r * ux / T(6);
+    const T ux = radd(T(-1), zh_div(fma_(T(2), radd(radd(f[1], f[5]), f[8]), radd(radd(f[0], f[2]), f[4])), r));
+    const T d = rsub(f[2], f[4]), q = rdiv(rmul(r, ux), T(6));
+    const T f3 = fma_(-rmul(T(2.0 / 3.0), r), ux, f[1]);
+    const T f7 = rsub(fma_(T(0.5), d, f[5]), q);
+    const T f6 = rsub(fma_(T(-0.5), d, f[8]), q);
     const T kR = fr[0] + fr[1] + fr[2] + fr[4] + fr[5] + fr[8];
     const T kT = f[0] + f[1] + f[2] + f[4] + f[5] + f[8];
     const T frac = kT != T(0) ? zh_div(kR, kT) : T(0);
-    fr[3] = frac * f3;
-    fb[3] = (T(1) - frac) * f3;
-    fr[6] = frac * f6;
-    fb[6] = (T(1) - frac) * f6;
-    fr[7] = frac * f7;
-    fb[7] = (T(1) - frac) * f7;
+    const T rest = rsub(T(1), frac);
+    fr[3] = rmul(frac, f3);
+    fb[3] = rmul(rest, f3);
+    fr[6] = rmul(frac, f6);
+    fb[6] = rmul(rest, f6);
+    fr[7] = rmul(frac, f7);
+    fb[7] = rmul(rest, f7);
   }
 }
 

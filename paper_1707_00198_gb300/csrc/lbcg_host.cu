@@ -631,6 +631,10 @@ lbcg_status lbcg_create_batch(int32_t n, const lbcg_geometry* geoms, const lbcg_
     d.grad_eps = p.grad_eps;
     d.h_inv_nuR = 0.5 / p.nu_R;
     d.h_inv_nuB = 0.5 / p.nu_B;
+    const LatConst<double> c = d.consts<double>();
+    d.cf = LatConst<float>{float(c.sigma),   float(c.beta),     float(c.s_e),       float(c.s_eps),
+                           float(c.s_q),     float(c.rho0),     float(c.u_in),      float(c.rho_out),
+                           float(c.grad_eps), float(c.h_inv_nuR), float(c.h_inv_nuB), float(c.cos_theta)};
   }
   h->node_total = node_total;
   h->flags_host.assign((size_t)node_total, F_SOLID);

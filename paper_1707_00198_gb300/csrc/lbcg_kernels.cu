@@ -16,6 +16,7 @@
 
 #include "lbcg_device.cuh"
 #include "lbcg_internal.h"
+#include "lbcg_node.cuh"
 
 namespace lbcg {
 
@@ -42,50 +43,12 @@ struct StepArgs {
 //      contact-angle correction of Eq. 30-36 -> corrected gradient and unit normal.
 // The arithmetic is rounding-exact in the oracle's order (directions 1..8, products w*phi
 // then sign); the host-built stencils only replace the flag lookups of that order.
-// Eq. 28 on an outermost fluid node from the shared values of its 8 neighbours, then
-// Eq. 30-36; writes the corrected gradient and unit normal.
+// Corrected gradient and unit normal of an outermost fluid node, written to the node arrays.
 template <typename T>
 __device__ __forceinline__ void wall_node(const LatDev& sL, const OfbEntry& e, const WallSten& q, const T* val,
                                           T* __restrict__ wall, long long node_total) {
-  T gx = T(0), gy = T(0);
-#pragma unroll
-  for (int a = 1; a < 9; ++a) {
-    const T tt = rmul(wgt<T>(a), val[q.i[a - 1]]);
-    if (ex(a) == 1) gx = radd(gx, tt);
-    if (ex(a) == -1) gx = radd(gx, -tt);
-    if (ey(a) == 1) gy = radd(gy, tt);
-    if (ey(a) == -1) gy = radd(gy, -tt);
-  }
-  const T cs2 = T(1.0 / 3.0);
-  gx = rdiv(gx, cs2);
-  gy = rdiv(gy, cs2);
-  const T eps = T(sL.grad_eps);
-  const T mag = rsqrt_(radd(rmul(gx, gx), rmul(gy, gy)));
-  T cgx = gx, cgy = gy, nx = T(0), ny = T(0);
-  if (mag > eps && sL.wetting == 2) {
-    nx = rdiv(gx, mag);   // no geometric correction: n from the raw gradient
-    ny = rdiv(gy, mag);
-  } else if (mag > eps) {
-    const T esx = rdiv(gx, mag), esy = rdiv(gy, mag);                 // Eq. 30
-    const T nsx = T(e.nsx), nsy = T(e.nsy), c = T(e.cos_t), s = T(e.sin_t);
-    const T f1x = rsub(rmul(nsx, c), rmul(nsy, s));                   // Eq. 34, +theta
-    const T f1y = radd(rmul(nsx, s), rmul(nsy, c));
-    const T f2x = radd(rmul(nsx, c), rmul(nsy, s));                   // Eq. 34, -theta
-    const T f2y = radd(rmul(-nsx, s), rmul(nsy, c));
-    const T a1 = rsub(f1x, esx), b1 = rsub(f1y, esy);
-    const T a2 = rsub(f2x, esx), b2 = rsub(f2y, esy);
-    const T d1 = rsqrt_(radd(rmul(a1, a1), rmul(b1, b1)));            // Eq. 35
-    const T d2 = rsqrt_(radd(rmul(a2, a2), rmul(b2, b2)));
-    const T nfx = d1 <= d2 ? f1x : f2x;                               // Eq. 36
-    const T nfy = d1 <= d2 ? f1y : f2y;
-    cgx = rmul(mag, nfx);                                             // Eq. 31
-    cgy = rmul(mag, nfy);
-    const T m2 = rsqrt_(radd(rmul(cgx, cgx), rmul(cgy, cgy)));
-    if (m2 > eps) {
-      nx = rdiv(cgx, m2);
-      ny = rdiv(cgy, m2);
-    }
-  }
+  T cgx, cgy, nx, ny;
+  wall_normal<T>(T(sL.grad_eps), sL.wetting, T(e.nsx), T(e.nsy), T(e.cos_t), T(e.sin_t), q, val, cgx, cgy, nx, ny);
   const long long k = sL.node_off + (long long)e.y * sL.pitch + e.x;
   wall[k] = cgx;
   wall[node_total + k] = cgy;
@@ -238,54 +201,13 @@ __global__ void __launch_bounds__(kWallThreads, sizeof(S) == 8 ? 3 : 5) k_wall(c
 }
 
 
-// Eq. 48, wetting scheme (b) (lbcg_params.wetting = 1): grad n at an outermost fluid node from
-// its fluid neighbours only, d_i n = sum_a w_a (n(x + e_a) - n(x)) e_ai / sum_a w_a e_ai^2 over
-// the directions a whose neighbour is fluid (bit a-1 of `solid` clear).  nxs/nys[a] hold n at
-// x + e_a (a = 0: the node).  Returned divided by 3 (= c_s^2): the bulk kernels keep their
-// Eq. 28 sums at that scale and apply 1/c_s^2 in the curvature.
-template <typename T>
-__device__ __forceinline__ void grad_n_scheme_b(const T nxs[9], const T nys[9], unsigned solid, T& dxx, T& dyx, T& dxy,
-                                                T& dyy) {
-  T sxx = T(0), syx = T(0), sxy = T(0), syy = T(0), wx = T(0), wy = T(0);
-#pragma unroll
-  for (int a = 1; a < 9; ++a) {
-    if ((solid >> (a - 1)) & 1u) continue;
-    const T w = wgt<T>(a), ddx = nxs[a] - nxs[0], ddy = nys[a] - nys[0];
-    if (ex(a)) {
-      sxx += T(ex(a)) * w * ddx;
-      syx += T(ex(a)) * w * ddy;
-      wx += w;
-    }
-    if (ey(a)) {
-      sxy += T(ey(a)) * w * ddx;
-      syy += T(ey(a)) * w * ddy;
-      wy += w;
-    }
-  }
-  const T third = T(1) / T(3);
-  dxx = wx > T(0) ? sxx / wx * third : T(0);
-  dyx = wx > T(0) ? syx / wx * third : T(0);
-  dxy = wy > T(0) ? sxy / wy * third : T(0);
-  dyy = wy > T(0) ? syy / wy * third : T(0);
-}
-
 // ------------------------------------------------------------------ k_step
-// Arithmetic helpers: the FP64 instantiation keeps IEEE divisions and square roots (it is the
-// validation path); the FP32-arithmetic instantiations use the hardware reciprocal and
-// reciprocal square root.
-template <typename T>
-__device__ __forceinline__ T rcp_(T x) {
-  if constexpr (sizeof(T) == 4) return __fdividef(1.0f, x);
-  else return T(1) / x;
-}
-
 // FP32-arithmetic instantiations are held to 64 registers so that 1024 threads fit on an
 // SM (they need no more); the FP64 validation instantiation keeps its registers.
 template <typename S, int TY, bool MACRO>
 __global__ void __launch_bounds__(32 * TY, sizeof(typename Store<S>::T) == 4 ? 1024 / (32 * TY) : 1)
     k_step(StepArgs A) {
   using T = typename Store<S>::T;
-  constexpr bool kF32 = sizeof(T) == 4;
   constexpr int TX = 32;
   constexpr int NT = TX * TY;
   constexpr int W3 = TX + 6, H3 = TY + 6;   // flags: tile + 3
@@ -308,7 +230,8 @@ __global__ void __launch_bounds__(32 * TY, sizeof(typename Store<S>::T) == 4 ? 1
   // lattice constants in registers (shared memory cannot alias the global stores below)
   const int nx = sL.nx, ny = sL.ny, pitch = sL.pitch;
   const bool px = sL.bcx == BC_PERIODIC, py = sL.bcy == BC_PERIODIC, inout = sL.bcx == BC_INOUT;
-  const T r0 = T(sL.rho0), u_in = T(sL.u_in), rho_out = T(sL.rho_out), eps = T(sL.grad_eps);
+  const LatConst<T> C = sL.consts<T>();
+  const T r0 = C.rho0, rho_out = C.rho_out, eps2 = rmul(C.grad_eps, C.grad_eps);
   const uint8_t* __restrict__ fl = A.flags + sL.node_off;
   const S* __restrict__ src = static_cast<const S*>(A.src) + sL.pop_off;
   const T* __restrict__ wall = static_cast<const T*>(A.wall) + sL.node_off;
@@ -336,30 +259,13 @@ __global__ void __launch_bounds__(32 * TY, sizeof(typename Store<S>::T) == 4 ? 1
     load_raw<S>(src + pop_node(x, sym[c3y], pitch), r0, fr_, fb_);
     if (inout) zou_he<T>(x, nx, inlet_u<T>(sL, sym[c3y]), rho_out, fr_, fb_);
   };
-  // rho^N (Eq. 12): exactly +-1 on single-colour nodes in both arithmetic paths
-  auto indicator = [&](const T fr_[9], const T fb_[9], T& sr, T& sb) -> T {
-    sr = fr_[0];
-    sb = fb_[0];
-#pragma unroll
-    for (int a = 1; a < 9; ++a) {
-      sr += fr_[a];
-      sb += fb_[a];
-    }
-    if constexpr (kF32) {
-      const T v = (sr - sb) * rcp_(sr + sb);
-      return sb == T(0) ? T(1) : (sr == T(0) ? T(-1) : v);
-    } else {
-      return (sr - sb) / (sr + sb);
-    }
-  };
-
   // ---- phase A: rho^N on tile + 2 (own node keeps its populations in registers)
   const int lx = tid % TX, ly = tid / TX;
-  T fr[9], fb[9], rhoR = T(0), rhoB = T(0), rn = T(0);
+  T fr[9], fb[9], rhoR = T(0), rhoB = T(0), rn = T(0), irho = T(0);
   const bool fluid = !(sfl[(ly + 3) * W3 + lx + 3] & F_SOLID);
   if (fluid) {
     load(lx + 3, ly + 3, fr, fb);
-    rn = indicator(fr, fb, rhoR, rhoB);
+    rn = indicator(fr, fb, rhoR, rhoB, irho);
   } else {
 #pragma unroll
     for (int a = 0; a < 9; ++a) fr[a] = fb[a] = T(0);
@@ -370,9 +276,9 @@ __global__ void __launch_bounds__(32 * TY, sizeof(typename Store<S>::T) == 4 ? 1
     if (cx >= 2 && cx < TX + 2 && cy >= 2 && cy < TY + 2) continue;
     T v = T(0);
     if (!(sfl[(cy + 1) * W3 + cx + 1] & F_SOLID)) {
-      T hr[9], hb[9], a1, a2;
+      T hr[9], hb[9], a1, a2, a3;
       load(cx + 1, cy + 1, hr, hb);
-      v = indicator(hr, hb, a1, a2);
+      v = indicator(hr, hb, a1, a2, a3);
     }
     srn[i] = v;
   }
@@ -409,29 +315,7 @@ __global__ void __launch_bounds__(32 * TY, sizeof(typename Store<S>::T) == 4 ? 1
         nxv = wall[2 * NTOT + k];
         nyv = wall[3 * NTOT + k];
       } else {
-        const int c2x = sx + 1, c2y = sy + 1;
-#pragma unroll
-        for (int a = 1; a < 9; ++a) {
-          const T t = wgt<T>(a) * srn[(c2y + ey(a)) * W2 + c2x + ex(a)];
-          if (ex(a)) ax += T(ex(a)) * t;
-          if (ey(a)) ay += T(ey(a)) * t;
-        }
-        ax *= T(3);
-        ay *= T(3);
-        const T m2 = ax * ax + ay * ay;
-        if constexpr (kF32) {
-          if (m2 > eps * eps) {
-            const T inv = rsqrtf(m2);
-            nxv = ax * inv;
-            nyv = ay * inv;
-          }
-        } else {
-          const T m = sqrt(m2);
-          if (m > eps) {
-            nxv = ax / m;
-            nyv = ay / m;
-          }
-        }
+        grad_normal<T>(srn + (sy + 1) * W2 + sx + 1, W2, eps2, ax, ay, nxv, nyv);
       }
     } else if (f & F_OSOLID) {
       // virtual n on the outermost solid node (Eq. 29); its fluid neighbours are outermost
@@ -442,14 +326,14 @@ __global__ void __launch_bounds__(32 * TY, sizeof(typename Store<S>::T) == 4 ? 1
         if (!(sfl[(c3y + ey(b)) * W3 + c3x + ex(b)] & F_SOLID)) {
           const int k2 = sym[c3y + ey(b)] * pitch + sxm[c3x + ex(b)];
           if (!checked(in_extent(k2, 1, sL.plane), A.err)) continue;
-          vx += wgt<T>(b) * wall[2 * NTOT + k2];
-          vy += wgt<T>(b) * wall[3 * NTOT + k2];
-          den += wgt<T>(b);
+          vx = fma_(wgt<T>(b), wall[2 * NTOT + k2], vx);
+          vy = fma_(wgt<T>(b), wall[3 * NTOT + k2], vy);
+          den = radd(den, wgt<T>(b));
         }
       }
       if (den > T(0)) {
-        nxv = vx / den;
-        nyv = vy / den;
+        nxv = rdiv(vx, den);
+        nyv = rdiv(vy, den);
       }
     }
     snx[cy * W1 + cx] = nxv;
@@ -465,21 +349,9 @@ __global__ void __launch_bounds__(32 * TY, sizeof(typename Store<S>::T) == 4 ? 1
   const int xs = x0 + lx, ys = y0 + ly;
   if (!fluid || xs >= nx || ys >= ny) return;
   const int c1x = lx + 1, c1y = ly + 1;
-  T dxx = T(0), dxy = T(0), dyx = T(0), dyy = T(0);  // d_x n_x, d_y n_x, d_x n_y, d_y n_y
-#pragma unroll
-  for (int a = 1; a < 9; ++a) {
-    const int o = (c1y + ey(a)) * W1 + c1x + ex(a);
-    const T tx = wgt<T>(a) * snx[o];
-    const T ty = wgt<T>(a) * sny[o];
-    if (ex(a)) {
-      dxx += T(ex(a)) * tx;
-      dyx += T(ex(a)) * ty;
-    }
-    if (ey(a)) {
-      dxy += T(ey(a)) * tx;
-      dyy += T(ey(a)) * ty;
-    }
-  }
+  const int o1 = c1y * W1 + c1x;
+  T dxx, dxy, dyx, dyy;  // d_x n_x, d_y n_x, d_x n_y, d_y n_y
+  grad_n<T>(snx + o1, sny + o1, W1, dxx, dyx, dxy, dyy);
   if (sL.wetting == 1 && (sfl[(ly + 3) * W3 + lx + 3] & F_OFB)) {
     T nxs[9], nys[9];
     unsigned solid = 0;
@@ -490,91 +362,44 @@ __global__ void __launch_bounds__(32 * TY, sizeof(typename Store<S>::T) == 4 ? 1
       nys[a] = sny[o];
       if (a && (sfl[(ly + 3 + ey(a)) * W3 + lx + 3 + ex(a)] & F_SOLID)) solid |= 1u << (a - 1);
     }
-    grad_n_scheme_b<T>(nxs, nys, solid, dxx, dyx, dxy, dyy);
+    grad_n_scheme_b<T>(nxs, nys, solid, kStencilScale<T>, dxx, dyx, dxy, dyy);
   }
-  const T nxo = snx[c1y * W1 + c1x], nyo = sny[c1y * W1 + c1x];
-  // Eq. 13 (the factor 3 = 1/c_s^2 of Eq. 28 applied once) and Eq. 10
-  const T kappa = T(3) * (-nxo * nxo * dyy - nyo * nyo * dxx + nxo * nyo * (dxy + dyx));
-  const T hsk = T(0.5) * T(sL.sigma) * kappa;
-  const T Fx = hsk * gx;
-  const T Fy = hsk * gy;
-
+  const T nxo = snx[o1], nyo = sny[o1];
   T f[9];
 #pragma unroll
-  for (int a = 0; a < 9; ++a) f[a] = fr[a] + fb[a];
-  const T rho = rhoR + rhoB;
-  const T irho = rcp_(rho);
-  const T jx = f[1] - f[3] + f[5] - f[6] - f[7] + f[8];
-  const T jy = f[2] - f[4] + f[5] + f[6] - f[7] - f[8];
-  const T ux = (jx + T(0.5) * Fx) * irho;                                         // Eq. 17
-  const T uy = (jy + T(0.5) * Fy) * irho;
+  for (int a = 0; a < 9; ++a) f[a] = radd(fr[a], fb[a]);
+  const Collide<T> K(C);
+  const T rho = radd(rhoR, rhoB);
+  Moments<T> m;
+  m.of(f);
+  T Fx, Fy;
+  csf_force<T>(gx, gy, nxo, nyo, dxx, dyx, dxy, dyy, K, Fx, Fy);
   const int kn = ys * pitch + xs;
   if constexpr (MACRO) {
     if (!checked(in_extent(kn, 1, sL.plane), A.err)) return;
     const long long k = sL.node_off + kn;
+    T ux, uy;
+    velocity<T>(m, irho, Fx, Fy, ux, uy);
     A.macro[k] = double(rhoR);
     A.macro[NTOT + k] = double(rhoB);
     A.macro[2 * NTOT + k] = double(ux);
     A.macro[3 * NTOT + k] = double(uy);
     return;
   } else {
-    // local viscosity (Eq. 18) and s_v = 1/tau_v = 1/(3 nu + 1/2) (Eq. 5)
-    const T inv_nu = (T(1) + rn) * T(sL.h_inv_nuR) + (T(1) - rn) * T(sL.h_inv_nuB);
-    const T sv = inv_nu * rcp_(T(3) + T(0.5) * inv_nu);
-    const T se = T(sL.s_e), seps = T(sL.s_eps), sq = T(sL.s_q);
-    // moments (rows of Eq. 3, the last one read as e_x e_y)
-    const T s14 = f[1] + f[2] + f[3] + f[4];
-    const T s58 = f[5] + f[6] + f[7] + f[8];
-    const T me = T(-4) * f[0] - s14 + T(2) * s58;
-    const T meps = T(4) * f[0] - T(2) * s14 + s58;
-    const T qx = T(-2) * (f[1] - f[3]) + (f[5] - f[6] - f[7] + f[8]);
-    const T qy = T(-2) * (f[2] - f[4]) + (f[5] + f[6] - f[7] - f[8]);
-    const T pxx = f[1] - f[2] + f[3] - f[4];
-    const T pxy = f[5] - f[6] + f[7] - f[8];
-    const T u2 = ux * ux + uy * uy;
-    const T uF = ux * Fx + uy * Fy;
-    // Delta_k = s_k (m_k - m_k^eq) - (1 - s_k/2) (M F~)_k  with M F~ =
-    // (0, 6 u.F, -6 u.F, Fx, -Fx, Fy, -Fy, 2(ux Fx - uy Fy), ux Fy + uy Fx)   (Eq. 8-9)
-    const T De = se * (me - rho * (T(-2) + T(3) * u2)) - (T(1) - T(0.5) * se) * (T(6) * uF);
-    const T Deps = seps * (meps - rho * (T(1) - T(3) * u2)) + (T(1) - T(0.5) * seps) * (T(6) * uF);
-    const T Dqx = sq * (qx + rho * ux) + (T(1) - T(0.5) * sq) * Fx;
-    const T Dqy = sq * (qy + rho * uy) + (T(1) - T(0.5) * sq) * Fy;
-    const T Dxx = sv * (pxx - rho * (ux * ux - uy * uy)) - (T(1) - T(0.5) * sv) * (T(2) * (ux * Fx - uy * Fy));
-    const T Dxy = sv * (pxy - rho * ux * uy) - (T(1) - T(0.5) * sv) * (ux * Fy + uy * Fx);
-    // M^-1 = M^T diag(1/9, 1/36, 1/36, 1/6, 1/12, 1/6, 1/12, 1/4, 1/4); s_rho = s_j = 1
-    // (Eq. 6), so the momentum rows give Delta_j = -F: the momentum changes by exactly F
-    const T ae = De * T(1.0 / 36.0), aeps = Deps * T(1.0 / 36.0);
-    const T ajx = -Fx * T(1.0 / 6.0), ajy = -Fy * T(1.0 / 6.0);
-    const T aqx = Dqx * T(1.0 / 12.0), aqy = Dqy * T(1.0 / 12.0);
-    const T axx = Dxx * T(0.25), axy = Dxy * T(0.25);
     T fp[9];
-    fp[0] = f[0] - (T(-4) * ae + T(4) * aeps);
-    const T c14 = -ae - T(2) * aeps;
-    fp[1] = f[1] - (c14 + ajx - T(2) * aqx + axx);
-    fp[2] = f[2] - (c14 + ajy - T(2) * aqy - axx);
-    fp[3] = f[3] - (c14 - ajx + T(2) * aqx + axx);
-    fp[4] = f[4] - (c14 - ajy + T(2) * aqy - axx);
-    const T c58 = T(2) * ae + aeps;
-    fp[5] = f[5] - (c58 + ajx + aqx + ajy + aqy + axy);
-    fp[6] = f[6] - (c58 - ajx - aqx + ajy + aqy - axy);
-    fp[7] = f[7] - (c58 - ajx - aqx - ajy - aqy + axy);
-    fp[8] = f[8] - (c58 + ajx + aqx - ajy - aqy - axy);
-    // recolouring (Eq. 14; the blue line with the minus sign)
-    const T cR = rhoR * irho, cB = rhoB * irho;
-    const T pc = T(sL.beta) * rhoR * rhoB * irho;
+    collide_node<T>(f, m, rho, irho, viscous_rate<T>(rn, K), Fx, Fy, K, fp);
+    const Recolour<T> rc(rhoR, rhoB, irho, nxo, nyo, K);
     S* __restrict__ dst = static_cast<S*>(A.dst) + sL.pop_off;
     uint32_t srk = 0;
-    if constexpr (Store<S>::kDeviation) srk = sr_key(A.sr_epoch, A.sr_step, sL.pop_off);
+    if constexpr (Store<S>::kDeviation) srk = sr_key(*A.sr_epoch, A.sr_step, sL.pop_off);
     const int c3x = lx + 3, c3y = ly + 3;
     const int pn_own = pop_node(xs, ys, pitch);
     uint32_t srh = 0;
     if constexpr (Store<S>::kDeviation) srh = sr_node(srk, pn_own);
 #pragma unroll
     for (int a = 0; a < 9; ++a) {
-      const T en = T(ex(a)) * nxo + T(ey(a)) * nyo;
-      const T pert = pc * wgt<T>(a) * en;
-      const T oR = cR * fp[a] + pert;
-      const T oB = cB * fp[a] - pert;
+      T oR, oB;
+      rc.out(a, fp, oR, oB);
       // streaming (Eq. 15): to x + e_a if that node is fluid; half-way bounce-back into the
       // opposite slot of this node if it is solid; dropped if it lies beyond an open edge
       int k = pn_own, slot = a;
@@ -855,7 +680,7 @@ __global__ void __launch_bounds__(NTH, sizeof(typename Store<S>::T) == 4 ? 1024 
         nxs[a] = v.x;
         nys[a] = v.y;
       }
-      grad_n_scheme_b<T>(nxs, nys, mask, dxx, dyx, dxy, dyy);
+      grad_n_scheme_b<T>(nxs, nys, mask, T(1) / T(3), dxx, dyx, dxy, dyy);
     }
     const T nxo = n0_c.x, nyo = n0_c.y;
     const T kappa = T(3) * (-nxo * nxo * dyy - nyo * nyo * dxx + nxo * nyo * (dxy + dyx));
@@ -1050,7 +875,7 @@ __global__ void __launch_bounds__(NTH, sizeof(S) == 4 ? kSweepFMinBlocks : kSwee
   const S* __restrict__ src = static_cast<const S*>(A.src) + sL.pop_off;
   S* __restrict__ dst = static_cast<S*>(A.dst) + sL.pop_off;
   uint32_t srk = 0;
-  if constexpr (Store<S>::kDeviation) srk = sr_key(A.sr_epoch, A.sr_step, sL.pop_off);
+  if constexpr (Store<S>::kDeviation) srk = sr_key(*A.sr_epoch, A.sr_step, sL.pop_off);
 
   const int cx = sp.y - 2 + t;
   const int xm = wrap_or_clamp(cx, nx, px);
@@ -1318,7 +1143,7 @@ __global__ void __launch_bounds__(NTH, sizeof(S) == 4 ? kSweepFMinBlocks : kSwee
           nxs[a] = v.x;
           nys[a] = v.y;
         }
-        grad_n_scheme_b<T>(nxs, nys, mask, dX.x, dX.y, dY.x, dY.y);
+        grad_n_scheme_b<T>(nxs, nys, mask, T(1) / T(3), dX.x, dX.y, dY.x, dY.y);
       }
     }
     const T nxo = n0_c.x, nyo = n0_c.y;
