@@ -170,8 +170,11 @@ lbcg_status lbcg_create(const lbcg_geometry* geom, const lbcg_params* prm, int32
 lbcg_status lbcg_create_batch(int32_t n, const lbcg_geometry* geoms, const lbcg_params* prms,
                               int32_t precision, void* stream, lbcg_handle** out);
 
-/* Enqueue `nsteps` >= 0 time steps on the handle's stream (asynchronous; replayed from a
- * captured CUDA graph when nsteps is large). */
+/* Enqueue `nsteps` >= 0 time steps on the handle's stream (asynchronous).  A call of more than 32
+ * steps of a handle on the tile schedule whose lattices fit on the GPU at once (one tile per
+ * resident block) is launched as one cooperative kernel that takes all the steps (at most 8192
+ * per launch); other calls of 32 steps and more replay a captured CUDA graph, and short ones
+ * launch each kernel.  The results do not depend on which. */
 lbcg_status lbcg_step(lbcg_handle* h, int64_t nsteps);
 
 /* Measure the observables of lattice `lattice` of the current state (synchronises the
@@ -222,7 +225,7 @@ lbcg_status lbcg_set_tile(lbcg_handle* h, int32_t ty);
  * record).  The checks change no arithmetic: a checked run that reports nothing produces the
  * same bits as the normal build.  The normal build compiles them out. */
 
-/* Failure detection of the y-sweep's only device-side wait.  In the FP32 and 16-bit y-sweep a
+/* Failure detection of the device-side waits.  In the FP32 and 16-bit y-sweep a
  * block stages each row in shared memory with bulk asynchronous copies that complete on an
  * mbarrier, and every thread waits for the row with a bounded number of polls (default 2^22,
  * about a second; a wait that healthy hardware always finishes in microseconds).  When a wait
@@ -233,7 +236,10 @@ lbcg_status lbcg_set_tile(lbcg_handle* h, int32_t ty);
  * the handle usable: the state of the steps since the previous check is unreliable and should
  * be replaced (lbcg_set_populations, lbcg_upload_state).  lbcg_set_poll_limit sets the number
  * of polls (polls < 0 restores the default; 0 makes every wait give up at once, which tests
- * the path without any fault).  Synchronises and drops captured graphs. */
+ * the path without any fault).  Synchronises and drops captured graphs.
+ * The cooperative kernel of long calls (lbcg_step) has the other device-side wait, of a tile for
+ * the tiles around it, always with the default bound and reported the same way; a handle whose
+ * limit was changed launches each kernel of its steps instead. */
 lbcg_status lbcg_set_poll_limit(lbcg_handle* h, int32_t polls);
 
 /* Gradients by the discrete adjoint (reverse mode) of the step.  From the handle's current
@@ -322,7 +328,8 @@ lbcg_status lbcg_kernel_times(lbcg_handle* h, double* ms2, int64_t* steps);
 /* Number of kernel launches one directly launched time step enqueues (the wall kernel and the
  * bulk kernel), the number of kernel launches lbcg_step has enqueued on the handle since it was
  * created (each kernel node of a replayed graph counts: a batch's graph runs its lattices as
- * up to 3 parallel branches of their own launches), and the number of lattice nodes (fluid and
+ * up to 3 parallel branches of their own launches; a cooperative launch of many steps is one,
+ * with 16-bit storage two), and the number of lattice nodes (fluid and
  * solid) all lattices hold. */
 int32_t lbcg_launches_per_step(const lbcg_handle* h);
 int64_t lbcg_step_launches(const lbcg_handle* h);

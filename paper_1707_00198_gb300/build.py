@@ -19,7 +19,8 @@ LIB = os.path.join(HERE, "liblbcg.so")
 BUILD_CHECKED = os.path.join(HERE, "_build_checked")
 LIB_CHECKED = os.path.join(HERE, "liblbcg_checked.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
-SOURCES = ("lbcg_host.cu", "lbcg_kernels.cu", "lbcg_obs.cu", "lbcg_noalloc.cu", "lbcg_adjoint.cu", "lbcg_geom.cpp")
+SOURCES = ("lbcg_host.cu", "lbcg_kernels.cu", "lbcg_run.cu", "lbcg_obs.cu", "lbcg_noalloc.cu", "lbcg_adjoint.cu",
+           "lbcg_geom.cpp", "lbcg_plan.cpp")
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 
 

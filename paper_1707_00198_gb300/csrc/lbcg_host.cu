@@ -42,10 +42,12 @@ lbcg_status fail(lbcg_status s, const char* fmt, ...) {
 std::mutex g_alloc_mutex;
 lbcg_allocator g_allocator = {nullptr, nullptr, nullptr};
 
-constexpr int kGraphSteps = 32;   // steps per captured graph (even: the graph starts and ends on pool A)
+constexpr int kGraphSteps = kReplaySteps;   // steps per captured graph (even: the graph starts and ends on pool A)
 constexpr int kGraphBranches = 3; // parallel branches of a batch's graph (groups of lattices)
 constexpr int kHostGroups = 8;    // lattice groups whose copies lbcg_step_host overlaps
 constexpr int kDefaultTY = 8;
+constexpr int kPollLimit = 1 << 22;   // default polls of a bounded device wait (about a second)
+constexpr int kRunMaxSteps = 8192;    // steps per launch of the resident kernel, at most
 constexpr int kSMs = 152;
 
 size_t elem_size(int prec) { return prec == 0 ? 8 : (prec == 1 ? 4 : 2); }
@@ -78,7 +80,7 @@ struct lbcg_handle {
   uint8_t* d_nbmask = nullptr;
   int scheme_b = 0;        // some lattice uses wetting scheme (b)
   int* d_err = nullptr;    // device error word (a sweep block's bounded wait ran out)
-  int poll_limit = 1 << 22;   // polls of a sweep block's wait for a staged row (about a second)
+  int poll_limit = kPollLimit;   // polls of a sweep block's wait for a staged row (about a second)
   uint32_t* d_sr_epoch = nullptr;     // 16-bit storage: graph replays so far (stochastic-rounding keys)
   double* d_usnap = nullptr;          // velocity stored by lbcg_diagnostics ([2][node_total])
   std::vector<int64_t> snap_step;     // per lattice: step of that velocity, -1 = none
@@ -99,6 +101,15 @@ struct lbcg_handle {
   OfbEntry* d_ofb = nullptr;
   int nofb = 0;
   double* d_obs = nullptr;   // partials then outputs
+  // the resident kernel of the tile schedule (calls of more than kGraphSteps steps): its plan
+  // on the device, or run_tiles = 0 where the lattices do not fit
+  bool run_planned = false;
+  int run_tiles = 0;
+  size_t run_smem = 0;
+  char* d_run = nullptr;          // the plan's lists, one after another
+  unsigned* d_progress = nullptr; // per tile: steps finished, counted from run_base
+  unsigned run_base = 0;
+  RunArgs run = {};               // the device pointers of a launch
   cudaGraphExec_t graph = nullptr;
   int64_t graph_kernels = 0;    // kernel nodes of the captured graph
   int64_t step_launches = 0;    // kernel launches lbcg_step has enqueued (graph nodes counted)
@@ -346,7 +357,8 @@ void free_handle(lbcg_handle* h) {
   if (h->prof_ref) cudaEventDestroy(h->prof_ref);
   void* ptrs[] = {h->pool[0], h->pool[1], h->d_flags,  h->d_wall,  h->d_macro, h->d_lats,
                   h->d_tiles, h->d_groups, h->d_wband, h->d_wvirt, h->d_wsten, h->d_ofb,
-                  h->d_obs,   h->d_strips, h->d_nbmask, h->d_err, h->d_usnap, h->d_sr_epoch};
+                  h->d_obs,   h->d_strips, h->d_nbmask, h->d_err, h->d_usnap, h->d_sr_epoch,
+                  h->d_run,   h->d_progress};
   if (h->stream) cudaStreamSynchronize(h->stream);
   for (void* p : ptrs) dev_free(h, p);
   for (int b = 0; b < kGraphBranches; ++b) {
@@ -407,6 +419,107 @@ lbcg_status upload_tiles(lbcg_handle* h) {
   return LBCG_OK;
 }
 
+// Plans the resident kernel and uploads the plan (once per handle, when the tile schedule is
+// chosen).  Lattices that do not fit keep the launch-per-step schedule.
+lbcg_status plan_run(lbcg_handle* h) {
+  if (h->run_planned) return LBCG_OK;
+  h->run_planned = true;
+  int dev = 0, sms = 0, smem_max = 0;
+  CK(h, cudaGetDevice(&dev));
+  CK(h, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  CK(h, cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  const size_t cs = compute_size(h->prec), budget = size_t(std::max(0, smem_max - 2048));   // static shared memory apart
+  std::vector<LatGeom> views;
+  std::vector<const uint8_t*> flags;
+  long long fluid = 0;
+  for (const LatHost& L : h->lats) {
+    views.push_back(LatGeom{L.nx, L.ny, L.pitch, L.bcx, L.bcy, L.solid.data()});
+    flags.push_back(&h->flags_host[L.node_off]);
+    fluid += L.n_fluid;
+  }
+  // (a fluid node takes at least its 12 values and 8 bytes of tables)
+  if (fluid * (long long)(12 * cs + 8) > (long long)sms * (long long)budget) return LBCG_OK;
+  RunPlan p;
+  if (!build_run_plan(views, flags, h->ofb_host, sms, budget, cs, p)) return LBCG_OK;
+  int per_sm = 0;
+  CK(h, prepare_run(h->prec, p.smem, &per_sm));
+  if ((long long)per_sm * sms < (long long)p.tiles.size()) return LBCG_OK;
+  size_t total = 0;
+  std::vector<std::pair<const void*, size_t>> parts;
+  std::vector<size_t> at;
+  auto add = [&](const void* src, size_t bytes) {
+    at.push_back(total);
+    parts.push_back({src, bytes});
+    total += (bytes + 255) & ~size_t(255);
+  };
+  add(p.tiles.data(), p.tiles.size() * sizeof(RunTile));
+  add(p.nb.data(), p.nb.size() * sizeof(int));
+  add(p.extra.data(), p.extra.size() * sizeof(int));
+  add(p.w_ofb.data(), p.w_ofb.size() * sizeof(int));
+  add(p.w_sten.data(), p.w_sten.size() * sizeof(WallSten));
+  add(p.v_sten.data(), p.v_sten.size() * sizeof(WallSten));
+  add(p.copies.data(), p.copies.size() * sizeof(uint32_t));
+  add(p.vn.data(), p.vn.size() * sizeof(RunVirtN));
+  std::vector<char> host(std::max<size_t>(total, 16), 0);
+  for (size_t i = 0; i < parts.size(); ++i)
+    if (parts[i].second) memcpy(host.data() + at[i], parts[i].first, parts[i].second);
+  const size_t pb = p.tiles.size() * kRunFlagStride * sizeof(unsigned);
+  if (!dev_alloc(h, (void**)&h->d_run, host.size()) || !dev_alloc(h, (void**)&h->d_progress, pb))
+    return fail(LBCG_E_NOMEM, "cannot allocate the plan of the resident kernel");
+  CK(h, cudaMemcpy(h->d_run, host.data(), host.size(), cudaMemcpyHostToDevice));
+  CK(h, cudaMemset(h->d_progress, 0, pb));
+  RunArgs a{};
+  a.lats = h->d_lats;
+  a.tiles = reinterpret_cast<const RunTile*>(h->d_run + at[0]);
+  a.nb = reinterpret_cast<const int*>(h->d_run + at[1]);
+  a.extra = reinterpret_cast<const int*>(h->d_run + at[2]);
+  a.w_ofb = reinterpret_cast<const int*>(h->d_run + at[3]);
+  a.w_sten = reinterpret_cast<const WallSten*>(h->d_run + at[4]);
+  a.v_sten = reinterpret_cast<const WallSten*>(h->d_run + at[5]);
+  a.copies = reinterpret_cast<const uint32_t*>(h->d_run + at[6]);
+  a.vn = reinterpret_cast<const RunVirtN*>(h->d_run + at[7]);
+  a.ofb = h->d_ofb;
+  a.flags = h->d_flags;
+  a.nbmask = h->d_nbmask;
+  a.progress = h->d_progress;
+  a.err = h->d_err;
+  a.poll_limit = kPollLimit;
+  a.sr_epoch = h->d_sr_epoch;
+  h->run = a;
+  h->run_smem = p.smem;
+  h->run_tiles = int(p.tiles.size());
+  return LBCG_OK;
+}
+
+// Whether a call of nsteps steps runs as launches of the resident kernel.  Calls of up to
+// kGraphSteps steps keep the launch-per-step schedule (the resident kernel's launch resolves the
+// lattice's tables first), and so do profiled handles (events around each kernel), handles
+// whose poll limit was changed and streams that are being captured.
+bool runs_resident(const lbcg_handle* h, int64_t nsteps) {
+  if (h->sweep || h->run_tiles == 0 || nsteps <= kGraphSteps || h->profiling || h->poll_limit != kPollLimit) return false;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(h->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+}
+
+// One launch of the resident kernel: n steps from the handle's current state; *n is lowered to
+// what one launch takes.
+cudaError_t enqueue_run(lbcg_handle* h, int64_t* n) {
+  const int pre = h->cur;   // graph replays start from pool 0
+  if (*n > kRunMaxSteps) *n = pre + kRunMaxSteps / kGraphSteps * kGraphSteps;
+  RunArgs a = h->run;
+  a.pool0 = static_cast<char*>(h->pool[h->cur]);
+  a.pool1 = static_cast<char*>(h->pool[h->cur ^ 1]);
+  a.nsteps = int(*n);
+  a.base = h->run_base;
+  a.step0 = uint32_t(h->step);
+  a.pre = pre;
+  a.nrep = int((*n - pre) / kGraphSteps);
+  h->run_base += unsigned(*n);
+  cudaError_t e = launch_run(h->prec, a, h->run_tiles, h->run_smem, h->stream);
+  if (e == cudaSuccess && h->prec >= 2 && a.nrep > 0) e = launch_sr_add(h->d_sr_epoch, uint32_t(a.nrep), h->stream);
+  return e;
+}
+
 lbcg_status ensure_macro(lbcg_handle* h) {
   if (!h->d_macro) {
     if (!dev_alloc(h, (void**)&h->d_macro, 4 * (size_t)h->node_total * sizeof(double)))
@@ -416,9 +529,9 @@ lbcg_status ensure_macro(lbcg_handle* h) {
   return LBCG_OK;
 }
 
-// After a synchronisation: a sweep block gave up waiting for a staged row, so the state of
-// the steps since the last check is unreliable (that block stopped without writing the rest
-// of its rows).  The word is cleared once reported: the handle stays usable, and a state set
+// After a synchronisation: a sweep block gave up waiting for a staged row (or a block of the
+// resident kernel for a tile next to it), so the state of the steps since the last check is
+// unreliable (that block stopped without writing the rest).  The word is cleared once reported: the handle stays usable, and a state set
 // or uploaded afterwards steps correctly again.
 lbcg_status check_device_error(lbcg_handle* h) {
   int e = 0;
@@ -431,7 +544,7 @@ lbcg_status check_device_error(lbcg_handle* h) {
       return fail(LBCG_E_BOUNDS, "a range check of the checked build failed in a step kernel (the access was "
                                  "skipped; the state since the last check is unreliable)");
     return fail(LBCG_E_TIMEOUT,
-                "a sweep kernel's bounded wait for a staged row ran out%s; the state since the last check is "
+                "a step kernel's bounded wait ran out%s; the state since the last check is "
                 "unreliable",
                 (e & ERR_DRAIN) ? " and its copies could not be drained" : "");
   }
@@ -716,6 +829,7 @@ lbcg_status lbcg_create_batch(int32_t n, const lbcg_geometry* geoms, const lbcg_
       h->sweep = 0;
       h->ty = precision == LBCG_FP64 ? 4 : kDefaultTY;
       s = upload_tiles(h);
+      if (s == LBCG_OK) s = plan_run(h);
     }
     if (s != LBCG_OK) {
       free_handle(h);
@@ -796,6 +910,15 @@ lbcg_status lbcg_step(lbcg_handle* h, int64_t nsteps) {
       h->cur ^= 1;
       h->step += 1;
       nsteps -= 1;
+      continue;
+    }
+    if (runs_resident(h, nsteps)) {
+      int64_t n = nsteps;
+      CK(h, enqueue_run(h, &n));
+      h->step_launches += h->prec >= 2 ? 2 : 1;
+      h->cur ^= int(n & 1);
+      h->step += n;
+      nsteps -= n;
       continue;
     }
     if (nsteps >= kGraphSteps && h->cur == 0) {
@@ -1515,7 +1638,7 @@ lbcg_status lbcg_set_sweep(lbcg_handle* h, int32_t rows) {
 lbcg_status lbcg_set_poll_limit(lbcg_handle* h, int32_t polls) {
   lbcg_status s = check_handle(h);
   if (s != LBCG_OK) return s;
-  if (polls < 0) polls = 1 << 22;
+  if (polls < 0) polls = kPollLimit;
   CK(h, cudaStreamSynchronize(h->stream));
   h->poll_limit = polls;
   if (h->graph) {
@@ -1537,7 +1660,8 @@ lbcg_status lbcg_set_tile(lbcg_handle* h, int32_t ty) {
     cudaGraphExecDestroy(h->graph);
     h->graph = nullptr;
   }
-  return upload_tiles(h);
+  s = upload_tiles(h);
+  return s == LBCG_OK ? plan_run(h) : s;
 }
 
 lbcg_status lbcg_autotune(lbcg_handle* h, int32_t probe_steps, int32_t* schedule) {

@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "lbcg_device.cuh"
+#include "lbcg_plan.h"
 
 namespace lbcg {
 
@@ -49,6 +50,50 @@ cudaError_t launch_sr_tick(uint32_t* epoch, cudaStream_t st);
 // One-time kernel attributes for a precision (the sweep's dynamic shared memory); called
 // before any launch or graph capture of that precision.
 cudaError_t prepare_kernels(int prec);
+
+// ---- the resident step kernel (lbcg_run.cu)
+constexpr int kRunFlagStride = 32;   // unsigned ints between the tiles' progress words (128 bytes)
+constexpr int kReplaySteps = 32;     // steps of one graph replay of the launch-per-step schedule
+// Steps 0 .. nsteps - 1 of one launch: step s reads state(s) and writes state(s + 1).
+struct RunArgs {
+  const LatDev* lats;
+  const RunTile* tiles;
+  const int *nb, *extra, *w_ofb;
+  const WallSten *w_sten, *v_sten;
+  const uint32_t* copies;
+  const RunVirtN* vn;
+  const OfbEntry* ofb;
+  const uint8_t* flags;
+  const uint8_t* nbmask;
+  char *pool0, *pool1;    // the states: pool0 and pool1 in turn (stride 0),
+  long long stride;       // or one after another from pool0, `stride` bytes apart
+  int nsteps;
+  unsigned* progress;     // per tile: base + the steps it has finished
+  unsigned base;
+  int* err;
+  int poll_limit;
+  // Stochastic rounding draws the keys of the launch-per-step schedule: `pre` direct steps,
+  // nrep graph replays of kReplaySteps steps, then direct steps (absolute step numbers from
+  // step0).  The launcher advances the replay counter by nrep afterwards.
+  const uint32_t* sr_epoch;
+  uint32_t step0;
+  int pre, nrep;
+  __device__ __forceinline__ char* state(int s) const {
+    if (stride) return pool0 + s * stride;
+    return (s & 1) ? pool1 : pool0;
+  }
+  __device__ __forceinline__ uint32_t key(uint32_t epoch, int s, long long pop_off) const {
+    const int q = s - pre;
+    if (q >= 0 && q < nrep * kReplaySteps)
+      return sr_key(epoch + 1u + uint32_t(q / kReplaySteps), uint32_t(q % kReplaySteps), pop_off);
+    return sr_key(q < 0 ? epoch : epoch + uint32_t(nrep), step0 + uint32_t(s), pop_off);
+  }
+};
+cudaError_t launch_run(int prec, const RunArgs& a, int ntiles, size_t smem, cudaStream_t st);
+// sets the kernel's shared memory and asks how many of its blocks an SM holds
+cudaError_t prepare_run(int prec, size_t smem, int* per_sm);
+cudaError_t launch_sr_add(uint32_t* epoch, uint32_t n, cudaStream_t st);
+
 cudaError_t launch_to_storage(int prec, const LatDev* lats, int lat, long long nn, const double* in,
                               const uint8_t* flags, void* pool, cudaStream_t st);
 cudaError_t launch_from_storage(int prec, const LatDev* lats, int lat, long long nn, const void* pool,

@@ -1,0 +1,113 @@
+"""The resident kernel of the tile schedule (calls of more than 32 steps): the same bits as one
+launch per kernel and step, in every storage form, on lattices where a tile's halo wraps, clamps
+or covers the whole lattice, on walls of every kind, open columns and batches."""
+import dataclasses
+import math
+
+import numpy as np
+import pytest
+
+from paper_1707_00198_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+
+def _porous(nx, ny, seed):
+    """Periodic box with random solid nodes (about a tenth)."""
+    rng = np.random.default_rng(seed)
+    g = I.periodic_box_droplet(nx, ny, R=0.3 * ny, noise=1e-3, seed=seed)
+    solid = (rng.random((ny, nx)) < 0.1).astype(np.uint8)
+    return dataclasses.replace(g, solid=solid)
+
+
+def _theta_node(g, seed):
+    rng = np.random.default_rng(seed)
+    return dataclasses.replace(g, theta_node=rng.uniform(0.6, 2.4, (g.ny, g.nx)))
+
+
+def _cases():
+    P = I.Params
+    finger = I.fingering_params(5.0, 0.1, 60.0)
+    yield "tiny periodic", [I.periodic_box_droplet(5, 5, R=1.6, noise=1e-2, seed=1)], [P(sigma=0.02)]
+    yield "one tile wide", [I.flat_wall_droplet(7, 40, R=3.0, noise=1e-2, seed=2)], [P(theta=1.0)]
+    yield "odd closed", [I.flat_wall_droplet(61, 33, R=14.0, seed=3, closed_x=True)], [P(theta=1.9, nu_B=0.05)]
+    yield "odd periodic", [I.periodic_box_droplet(97, 45, R=15.0, noise=1e-3, seed=4)], [P(sigma=0.02)]
+    yield "porous", [_porous(67, 50, 5)], [P(theta=0.8)]
+    yield "cylinder", [I.cylinder_droplet(60, 50, Rs=10.0, cx=30.0, cy=18.0, Rd=9.0, theta=1.9, noise=1e-3, seed=6)], \
+        [P(theta=1.9, sigma=0.02)]
+    yield "angle per node", [_theta_node(I.flat_wall_droplet(64, 30, R=12.0, seed=7), 8)], [P()]
+    yield "channel", [I.displacement_channel(W=21, L=115, x_I=25.0, seed=9, noise=1e-3)], [finger]
+    yield "Poiseuille channel", [I.displacement_channel(W=20, L=110, x_I=25.0, seed=10)], \
+        [dataclasses.replace(finger, inlet_profile=1)]
+    for w in (1, 2):
+        yield f"wetting {w}", [I.flat_wall_droplet(50, 30, R=12.0, seed=11)], [P(theta=1.2, wetting=w)]
+    yield "capillary", [I.capillary_filling(L=60, d=20, reservoir=31, wall=7, red_into=20, noise=1e-3, seed=12)], [P(theta=0.6)]
+    yield "batch", [I.displacement_channel(W=20, L=110, x_I=25.0, seed=13), I.periodic_box_droplet(33, 40, R=9.0, seed=14),
+                    I.flat_wall_droplet(48, 20, R=8.0, seed=15)], [finger, P(nu_B=0.05), P(theta=1.2)]
+
+
+CASES = list(_cases())
+
+
+def _handles(gs, ps, prec, n=2):
+    from paper_1707_00198_gb300.lbcg import Lattice
+    out = [Lattice(gs, ps, prec) for _ in range(n)]
+    for L in out:
+        L.set_tile(8)
+    return out
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("name,gs,ps", CASES, ids=[c[0] for c in CASES])
+def test_resident_steps_equal_single_steps(name, gs, ps, prec):
+    A, B = _handles(gs, ps, prec)
+    for _ in range(70):
+        A.step(1)
+    B.step(70)
+    assert B.step_launches == 1 and A.step_launches == 70 * A.launches_per_step
+    B.step(1)      # from the other pool, then again
+    B.step(41)
+    for _ in range(42):
+        A.step(1)
+    for i in range(len(gs)):
+        b = B.populations(i)
+        assert np.isfinite(b).all()
+        assert np.array_equal(A.populations(i), b), (name, prec, i)
+    A.close()
+    B.close()
+
+
+@pytest.mark.parametrize("prec", ["fp16", "bf16"])
+@pytest.mark.parametrize("name,gs,ps", CASES, ids=[c[0] for c in CASES])
+def test_resident_16bit_steps_draw_the_keys_of_graph_replays(name, gs, ps, prec):
+    # calls of 32 steps are graph replays of one launch per kernel and step; a call of 65 steps
+    # draws the keys of two replays and a direct step, also when it starts with a direct step
+    A, B = _handles(gs, ps, prec)
+    for n in (32, 32, 1, 1, 32, 2):
+        A.step(n)
+    B.step(65)
+    B.step(35)     # starts from the other pool: one direct step, a replay, two direct steps
+    for i in range(len(gs)):
+        assert np.array_equal(A.populations(i), B.populations(i)), (name, prec, i)
+    A.close()
+    B.close()
+
+
+def test_long_call_and_configuration_sizes():
+    # several launches of one call, and the tiles of the configurations' lattices
+    (A, B) = _handles([I.flat_wall_droplet(20, 12, R=5.0, seed=1)], [I.Params(theta=math.radians(70))], "fp32")
+    A.step(9001)
+    for _ in range(300):
+        B.step(30)
+    B.step(1)
+    assert A.step_launches == 2
+    assert np.array_equal(A.populations(), B.populations())
+    for g, p in (I.config_capillary(), I.config_fingering(M=5.0)):
+        A, B = _handles([g], [p], "fp32")
+        A.step(64)
+        B.step(32)
+        B.step(32)
+        assert A.step_launches == 1
+        assert np.array_equal(A.populations(), B.populations()), g.name
+        A.close()
+        B.close()
