@@ -277,12 +277,14 @@ typedef struct {
 lbcg_status lbcg_adjoint(lbcg_handle* h, const lbcg_adjoint_spec* spec, lbcg_grads* out);
 
 /* Schedule of the step kernel.  lbcg_create picks the y-sweep over 124-column strips when
- * the strips give each of the 152 SMs a block, else 32-wide tiles (height 4 for FP64,
+ * the strips give each of the 152 SMs a block (FP64: and the lattices are too large for the
+ * cooperative kernel of long calls, see lbcg_step), else 32-wide tiles (height 4 for FP64,
  * 8 otherwise); lbcg_set_sweep / lbcg_set_tile choose one explicitly.  lbcg_autotune times
  * each candidate (the sweep with automatic segments and with segments of 24, 32, 40, 48, 56,
  * 64 and 80 rows; tiles 4, 8, 16) as lbcg_step runs it, a captured graph of `probe_steps`
  * steps (with a batch's parallel branches) that rewrite the same next state from the current
- * one without advancing it, keeps the fastest and writes it to *schedule (0 = sweep, else the tile height;
+ * one without advancing it, and the tiles as the cooperative kernel of long calls (the state is
+ * saved and put back), keeps the fastest and writes it to *schedule (0 = sweep, else the tile height;
  * schedule may be NULL).  It synchronises the handle's stream.  The candidates
  * give the same result up to rounding order (FP32: a few ulp per step; FP64 within 1e-13).
  * lbcg_schedule reports the current choice with the same encoding, lbcg_sweep_rows the

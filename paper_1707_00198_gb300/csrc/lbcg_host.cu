@@ -428,7 +428,9 @@ lbcg_status plan_run(lbcg_handle* h) {
   CK(h, cudaGetDevice(&dev));
   CK(h, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   CK(h, cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  const size_t cs = compute_size(h->prec), budget = size_t(std::max(0, smem_max - 2048));   // static shared memory apart
+  const size_t cs = compute_size(h->prec);
+  const int blocks = run_blocks(cs);
+  const size_t budget = size_t(std::max(0, smem_max / blocks - 2048));   // static and reserved shared memory apart
   std::vector<LatGeom> views;
   std::vector<const uint8_t*> flags;
   long long fluid = 0;
@@ -438,9 +440,9 @@ lbcg_status plan_run(lbcg_handle* h) {
     fluid += L.n_fluid;
   }
   // (a fluid node takes at least its 12 values and 8 bytes of tables)
-  if (fluid * (long long)(12 * cs + 8) > (long long)sms * (long long)budget) return LBCG_OK;
+  if (fluid * (long long)(12 * cs + 8) > (long long)sms * blocks * (long long)budget) return LBCG_OK;
   RunPlan p;
-  if (!build_run_plan(views, flags, h->ofb_host, sms, budget, cs, p)) return LBCG_OK;
+  if (!build_run_plan(views, flags, h->ofb_host, blocks * sms, budget, cs, p)) return LBCG_OK;
   int per_sm = 0;
   CK(h, prepare_run(h->prec, p.smem, &per_sm));
   if ((long long)per_sm * sms < (long long)p.tiles.size()) return LBCG_OK;
@@ -460,6 +462,7 @@ lbcg_status plan_run(lbcg_handle* h) {
   add(p.v_sten.data(), p.v_sten.size() * sizeof(WallSten));
   add(p.copies.data(), p.copies.size() * sizeof(uint32_t));
   add(p.vn.data(), p.vn.size() * sizeof(RunVirtN));
+  add(p.band.data(), p.band.size() * sizeof(uint16_t));
   std::vector<char> host(std::max<size_t>(total, 16), 0);
   for (size_t i = 0; i < parts.size(); ++i)
     if (parts[i].second) memcpy(host.data() + at[i], parts[i].first, parts[i].second);
@@ -478,6 +481,7 @@ lbcg_status plan_run(lbcg_handle* h) {
   a.v_sten = reinterpret_cast<const WallSten*>(h->d_run + at[5]);
   a.copies = reinterpret_cast<const uint32_t*>(h->d_run + at[6]);
   a.vn = reinterpret_cast<const RunVirtN*>(h->d_run + at[7]);
+  a.band = reinterpret_cast<const uint16_t*>(h->d_run + at[8]);
   a.ofb = h->d_ofb;
   a.flags = h->d_flags;
   a.nbmask = h->d_nbmask;
@@ -824,8 +828,11 @@ lbcg_status lbcg_create_batch(int32_t n, const lbcg_geometry* geoms, const lbcg_
   {
     lbcg_status s = upload_tiles(h);
     // default schedule: the y-sweep when its strips give every SM a block, else tiles
-    // (FP64 arithmetic is slow per SM, so FP64 takes the smallest tiles, i.e. the most blocks)
-    if (s == LBCG_OK && h->nstrips < kSMs) {
+    // (FP64 arithmetic is slow per SM, so FP64 takes the smallest tiles, i.e. the most blocks).
+    // FP64 lattices that the resident kernel holds take the tiles in any case: 2000 x 102,
+    // 248 us per step swept, 123 resident.
+    if (s == LBCG_OK && h->nstrips >= kSMs && precision == LBCG_FP64) s = plan_run(h);
+    if (s == LBCG_OK && (h->nstrips < kSMs || (precision == LBCG_FP64 && h->run_tiles > 0))) {
       h->sweep = 0;
       h->ty = precision == LBCG_FP64 ? 4 : kDefaultTY;
       s = upload_tiles(h);
@@ -1677,7 +1684,8 @@ lbcg_status lbcg_autotune(lbcg_handle* h, int32_t probe_steps, int32_t* schedule
   }
   // the y-sweep at the automatic segment height and at fixed heights, then the tiles; each
   // timed as what lbcg_step replays: a captured graph of probe_steps steps (with a batch's
-  // parallel branches), whose steps all rewrite the same next state
+  // parallel branches), whose steps all rewrite the same next state; last the tiles as one launch
+  // of the resident kernel
   struct Cand {
     int sweep, ty, rows;
   };
@@ -1688,8 +1696,8 @@ lbcg_status lbcg_autotune(lbcg_handle* h, int32_t probe_steps, int32_t* schedule
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   CK(h, cudaEventCreate(&e0));
   cudaError_t e = cudaEventCreate(&e1);
-  int best = 0;
-  float best_ms = 0.f;
+  int best = 0, best_tile = -1;
+  float best_ms = 0.f, tile_ms = 0.f;
   for (int c = 0; c < ncand && e == cudaSuccess; ++c) {
     h->sweep = cand[c].sweep;
     h->ty = cand[c].ty;
@@ -1712,6 +1720,40 @@ lbcg_status lbcg_autotune(lbcg_handle* h, int32_t probe_steps, int32_t* schedule
       best = c;
       best_ms = ms;
     }
+    if (e == cudaSuccess && !cand[c].sweep && (best_tile < 0 || ms < tile_ms)) {
+      best_tile = c;
+      tile_ms = ms;
+    }
+  }
+  // the tile schedule's resident kernel, where it applies: it advances the state, which is
+  // saved and put back
+  if (e == cudaSuccess && s == LBCG_OK) s = plan_run(h);
+  if (e == cudaSuccess && s == LBCG_OK && h->run_tiles > 0) {
+    const size_t sb = lbcg_state_bytes(h);
+    void* keep[2] = {nullptr, nullptr};
+    if (dev_alloc(h, &keep[0], sb) && dev_alloc(h, &keep[1], sb)) {
+      const int n = std::max(probe_steps, kGraphSteps + 1);
+      for (int q = 0; q < 2 && e == cudaSuccess; ++q)
+        e = cudaMemcpyAsync(keep[q], h->pool[q], sb, cudaMemcpyDeviceToDevice, h->stream);
+      RunArgs a = h->run;
+      a.pool0 = static_cast<char*>(h->pool[h->cur]);
+      a.pool1 = static_cast<char*>(h->pool[h->cur ^ 1]);
+      a.nsteps = n;
+      for (int q = 0; q < 2 && e == cudaSuccess; ++q) {
+        if (q) e = cudaEventRecord(e0, h->stream);
+        a.base = h->run_base;
+        h->run_base += unsigned(n);
+        if (e == cudaSuccess) e = launch_run(h->prec, a, h->run_tiles, h->run_smem, h->stream);
+      }
+      if (e == cudaSuccess) e = cudaEventRecord(e1, h->stream);
+      for (int q = 0; q < 2 && e == cudaSuccess; ++q)
+        e = cudaMemcpyAsync(h->pool[q], keep[q], sb, cudaMemcpyDeviceToDevice, h->stream);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+      float ms = 0.f;
+      if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+      if (e == cudaSuccess && ms / n < best_ms / probe_steps) best = best_tile;
+    }
+    for (void* q : keep) dev_free(h, q);
   }
   cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);

@@ -59,6 +59,7 @@ struct RunArgs {
   const LatDev* lats;
   const RunTile* tiles;
   const int *nb, *extra, *w_ofb;
+  const uint16_t* band;
   const WallSten *w_sten, *v_sten;
   const uint32_t* copies;
   const RunVirtN* vn;

@@ -3,16 +3,15 @@
 
 #include <algorithm>
 #include <cmath>
-#include <unordered_map>
 
 namespace lbcg {
 
 size_t run_smem_bytes(const RunTile& t, size_t cs) {
   auto up = [](size_t b) { return (b + 15) & ~size_t(15); };
   const size_t nr = size_t(t.tx + 4) * (t.ty + 4) + t.ne, np = size_t(t.tx + 2) * (t.ty + 2), no = size_t(t.tx) * t.ty;
-  return up(nr * cs) + up((nr + t.nv) * cs) + 4 * up(np * cs) + up(12 * no * cs) + up(8 * size_t(t.nw) * cs) +
+  return up(nr * cs) + up((size_t(t.nband) + t.nv) * cs) + 4 * up(np * cs) + up(12 * no * cs) + up(8 * size_t(t.nw) * cs) +
          up((size_t(t.nv) + t.nvn) * cs) +
-         up(nr * 4) * 2 + up((size_t(t.ty) + 8) * cs) + up(np * 2) + up(no * 8) + up((size_t(t.tx) + 2) * 4) + up((size_t(t.ty) + 2) * 4) +
+         up(nr * 4) * 2 + up(nr * 2) + up((size_t(t.ty) + 8) * cs) + up(np * 2) + up(no * 4) + up((size_t(t.tx) + 2) * 4) + up((size_t(t.ty) + 2) * 4) +
          up(t.nw * sizeof(WallSten)) + up(t.nv * sizeof(WallSten)) + up(t.nvn * sizeof(RunVirtN)) +
          up(size_t(t.ncopy) * 4);
 }
@@ -54,47 +53,64 @@ bool build_run_plan(const std::vector<LatGeom>& lats, const std::vector<const ui
   // (whole 32-byte sectors of the population rows) and n per slot of the ring around it weigh
   // about 6 : 1.2 : 1 in both arithmetics' instructions
   auto columns = [](int n, int side) { return (n + side - 1) / side; };
-  struct Eval {
-    long long count;
-    double cost;
-  };
-  auto eval = [&](int tx, int ty, long long limit) {
-    Eval e{0, 0.0};
-    for (int l = 0; l < nl && e.count <= limit; ++l) {
+  long long fluid = 0;
+  int nxmax = 1, nymax = 1;
+  for (int l = 0; l < nl; ++l) {
+    nxmax = std::max(nxmax, lats[l].nx);
+    nymax = std::max(nymax, lats[l].ny);
+    fluid += area[l].fluid(0, 0, lats[l].nx, lats[l].ny);
+  }
+  // f(lattice, x0, y0, x1, y1, fluid nodes) on every tile that has any; false once f is
+  auto each = [&](int tx, int ty, auto f) {
+    for (int l = 0; l < nl; ++l) {
       const int gx = columns(lats[l].nx, tx), gy = columns(lats[l].ny, ty);
-      for (int j = 0; j < gy && e.count <= limit; ++j)
-        for (int i = 0; i < gx; ++i) {
-          const int x0 = cut(lats[l].nx, gx, i), x1 = cut(lats[l].nx, gx, i + 1);
-          const int y0 = cut(lats[l].ny, gy, j), y1 = cut(lats[l].ny, gy, j + 1);
+      for (int j = 0; j < gy; ++j) {
+        const int y0 = cut(lats[l].ny, gy, j), y1 = cut(lats[l].ny, gy, j + 1);
+        for (int i = 0, x0 = 0; i < gx; ++i) {
+          const int x1 = cut(lats[l].nx, gx, i + 1);
           const int own = area[l].fluid(x0, y0, x1, y1);
-          if (own == 0) continue;
-          ++e.count;
-          const int hx0 = std::max(x0 - 2, 0), hy0 = std::max(y0 - 2, 0);
-          const int hx1 = std::min(x1 + 2, lats[l].nx), hy1 = std::min(y1 + 2, lats[l].ny);
-          const double halo = area[l].fluid(hx0, hy0, hx1, hy1) + 3.0 * (hy1 - hy0);
-          e.cost = std::max(e.cost, 6.0 * own + 1.2 * halo + double(x1 - x0 + 2) * (y1 - y0 + 2));
+          if (own && !f(l, x0, y0, x1, y1, own)) return false;
+          x0 = x1;
         }
+      }
     }
-    return e;
+    return true;
+  };
+  auto few = [&](int tx, int ty) {
+    int n = 0;
+    return each(tx, ty, [&](int, int, int, int, int, int) { return ++n <= max_tiles; });
+  };
+  auto cost = [&](int tx, int ty, double limit) {   // of the largest tile; `limit` or more: not measured to the end
+    double c = 0.0;
+    each(tx, ty, [&](int l, int x0, int y0, int x1, int y1, int own) {
+      const int hx0 = std::max(x0 - 2, 0), hy0 = std::max(y0 - 2, 0);
+      const int hx1 = std::min(x1 + 2, lats[l].nx), hy1 = std::min(y1 + 2, lats[l].ny);
+      const double halo = area[l].fluid(hx0, hy0, hx1, hy1) + 3.0 * (hy1 - hy0);
+      c = std::max(c, 6.0 * own + 1.2 * halo + double(x1 - x0 + 2) * (y1 - y0 + 2));
+      return c < limit;
+    });
+    return c;
   };
   int btx = 0, bty = 0;
-  double best = 0.0;
-  int nxmax = 1, nymax = 1;
-  for (const LatGeom& L : lats) {
-    nxmax = std::max(nxmax, L.nx);
-    nymax = std::max(nymax, L.ny);
-  }
-  for (int tx = 4; tx <= std::min(kRunMaxSide, std::max(4, nxmax)); tx += tx < 48 ? 1 : (tx < 96 ? 4 : 16)) {
-    int lo = 1, hi = std::min(kRunMaxSide, nymax);
-    if (eval(tx, hi, max_tiles).count > max_tiles) continue;
+  double best = 1e300;
+  for (int tx = 4; tx <= std::min(kRunMaxSide, std::max(4, nxmax)); tx += tx < 16 ? 1 : (tx < 48 ? 2 : (tx < 96 ? 4 : 16))) {
+    // a tile holds at most tx * ty fluid nodes: no height below lo can do
+    const int top = std::min(kRunMaxSide, nymax);
+    int lo = int(std::min<long long>(top, std::max<long long>(1, fluid / ((long long)max_tiles * tx))));
+    int hi = std::min(top, lo + lo / 4 + 2);
+    while (!few(tx, hi) && hi < top) {
+      lo = hi + 1;
+      hi = std::min(top, 2 * hi);
+    }
+    if (hi == top && !few(tx, hi)) continue;
     while (lo < hi) {
       const int mid = (lo + hi) / 2;
-      if (eval(tx, mid, max_tiles).count <= max_tiles) hi = mid;
+      if (few(tx, mid)) hi = mid;
       else lo = mid + 1;
     }
-    const Eval e = eval(tx, lo, max_tiles);
-    if (e.count <= max_tiles && (btx == 0 || e.cost < best)) {
-      best = e.cost;
+    const double c = cost(tx, lo, best);
+    if (c < best) {
+      best = c;
       btx = tx;
       bty = lo;
     }
@@ -108,7 +124,9 @@ bool build_run_plan(const std::vector<LatGeom>& lats, const std::vector<const ui
     const bool px = L.bcx == 0, py = L.bcy == 0;
     const int gx = columns(nx, btx), gy = columns(ny, bty);
     auto solid = [&](int x, int y) { return L.solid[size_t(y) * nx + x] != 0; };
-    std::unordered_map<int, int> ofb_at;   // node -> index in the outermost-fluid list
+    // per node: its index in the outermost-fluid list; and for the tile in hand, its index in w
+    // or among the virtual nodes (valid where the stamp is the tile's)
+    std::vector<int> ofb_at(size_t(nx) * ny), local(size_t(nx) * ny), stamp(size_t(nx) * ny, -1);
     for (; first_ofb < ofb.size() && ofb[first_ofb].lat == l; ++first_ofb)
       ofb_at[ofb[first_ofb].y * nx + ofb[first_ofb].x] = int(first_ofb);
     std::vector<int> col(nx), row(ny), id(size_t(gx) * gy, -1);
@@ -129,32 +147,39 @@ bool build_run_plan(const std::vector<LatGeom>& lats, const std::vector<const ui
         id[size_t(j) * gx + i] = int(plan.tiles.size());
         plan.tiles.push_back(t);
       }
-    std::vector<int> near;
+    std::vector<int> near, cols, rows;
+    // the columns (rows) of tiles that hold a node within kRunReach of [a, b)
+    auto reach = [&](int a, int b, int n, bool periodic, const std::vector<int>& of, std::vector<int>& out) {
+      out.clear();
+      for (int v = a - kRunReach; v < b + kRunReach; ++v) {
+        if (!periodic && (v < 0 || v >= n)) continue;
+        const int q = of[wrap_clamp(v, n, periodic)];
+        if (out.empty() || out.back() != q) out.push_back(q);
+        if (v == a) v = b - 1;   // inside [a, b) there is one
+      }
+      std::sort(out.begin(), out.end());
+      out.erase(std::unique(out.begin(), out.end()), out.end());
+    };
     for (size_t k = base; k < plan.tiles.size(); ++k) {
       RunTile& t = plan.tiles[k];
       near.clear();
-      for (int y = t.y0 - kRunReach; y < t.y0 + t.ty + kRunReach; ++y) {
-        if (!py && (y < 0 || y >= ny)) continue;
-        for (int x = t.x0 - kRunReach; x < t.x0 + t.tx + kRunReach; ++x) {
-          if (!px && (x < 0 || x >= nx)) continue;
-          // only the rim can hold another tile
-          if (y >= t.y0 && y < t.y0 + t.ty && x >= t.x0 && x < t.x0 + t.tx) {
-            x = t.x0 + t.tx - 1;
-            continue;
-          }
-          const int q = id[size_t(row[wrap_clamp(y, ny, py)]) * gx + col[wrap_clamp(x, nx, px)]];
-          if (q >= 0 && q != int(k) && (near.empty() || near.back() != q)) near.push_back(q);
+      reach(t.x0, t.x0 + t.tx, nx, px, col, cols);
+      reach(t.y0, t.y0 + t.ty, ny, py, row, rows);
+      for (int j : rows)
+        for (int i : cols) {
+          const int q = id[size_t(j) * gx + i];
+          if (q >= 0 && q != int(k)) near.push_back(q);
         }
-      }
-      std::sort(near.begin(), near.end());
-      near.erase(std::unique(near.begin(), near.end()), near.end());
       t.nb0 = int(plan.nb.size());
       t.nnb = int(near.size());
       plan.nb.insert(plan.nb.end(), near.begin(), near.end());
       // slots: the dense ones by position, the extra ones as they are asked for
       const int cw = t.tx + 4, ch = t.ty + 4, nd = cw * ch;
-      std::unordered_map<int, int> extra, wmap, vmap;
+      std::vector<int> extra;                          // nodes of the extra slots
+      std::vector<uint16_t> band_of(size_t(nd), kWallNone), band_of_extra;
+      int nw = 0, nband = 0;
       t.extra0 = int(plan.extra.size());
+      t.band0 = int(plan.band.size());
       t.w0 = int(plan.w_ofb.size());
       t.v0 = int(plan.v_sten.size());
       t.copy0 = int(plan.copies.size());
@@ -168,24 +193,43 @@ bool build_run_plan(const std::vector<LatGeom>& lats, const std::vector<const ui
       auto slot = [&](int x, int y) {   // of a fluid node of the lattice
         const int cx = inside(x - t.x0 + 2, nx, px, cw), cy = inside(y - t.y0 + 2, ny, py, ch);
         if (cx >= 0 && cy >= 0) return cy * cw + cx;
-        const auto it = extra.emplace(y * nx + x, nd + int(extra.size()));
-        if (it.second) plan.extra.push_back(y * nx + x);
-        return it.first->second;
+        const int node = y * nx + x;
+        for (size_t i = 0; i < extra.size(); ++i)
+          if (extra[i] == node) return nd + int(i);
+        extra.push_back(node);
+        band_of_extra.push_back(kWallNone);
+        plan.extra.push_back(node);
+        return nd + int(extra.size()) - 1;
+      };
+      auto in_band = [&](int x, int y) {
+        const int i = slot(x, y);
+        uint16_t& b = i < nd ? band_of[i] : band_of_extra[i - nd];
+        if (b == kWallNone) {
+          b = uint16_t(nband++);
+          plan.band.push_back(uint16_t(i));
+        }
+        return b;
       };
       auto want_w = [&](int x, int y) {   // of an outermost fluid node of the lattice
-        const auto it = wmap.emplace(y * nx + x, int(wmap.size()));
-        if (it.second) plan.w_ofb.push_back(ofb_at.at(y * nx + x));
-        return it.first->second;
+        const size_t n = size_t(y) * nx + x;
+        if (stamp[n] != int(k)) {
+          stamp[n] = int(k);
+          local[n] = nw++;
+          plan.w_ofb.push_back(ofb_at[n]);
+        }
+        return local[n];
       };
       const uint8_t* fl = flags[l];
-      for (int cy = 0; cy < t.ty + 2; ++cy)
+      for (int cy = 0; cy < t.ty + 2; ++cy) {
+        const int y = wrap_clamp(t.y0 + cy - 1, ny, py);
         for (int cx = 0; cx < t.tx + 2; ++cx) {
-          const int x = wrap_clamp(t.x0 + cx - 1, nx, px), y = wrap_clamp(t.y0 + cy - 1, ny, py);
+          const int xr = t.x0 + cx - 1, x = xr >= 0 && xr < nx ? xr : wrap_clamp(xr, nx, px);
           const uint8_t f = fl[size_t(y) * L.pitch + x];
+          if (!(f & (F_OFB | F_OSOLID))) continue;
           const uint32_t pos = uint32_t(cy * (t.tx + 2) + cx);
           if (f & F_OFB) {
             plan.copies.push_back(pos | uint32_t(want_w(x, y)) << 16);
-          } else if (f & F_OSOLID) {
+          } else {
             RunVirtN v{};
             v.pos = pos;
             for (int b = 1; b < 9; ++b) {
@@ -195,8 +239,9 @@ bool build_run_plan(const std::vector<LatGeom>& lats, const std::vector<const ui
             plan.vn.push_back(v);
           }
         }
-      // stencils of the outermost fluid nodes; virtual nodes are numbered after every slot, so
-      // their indices are fixed up once the extra slots are known
+      }
+      // stencils of the outermost fluid nodes; virtual nodes are numbered after the band, so
+      // their indices are fixed up once the band is known
       std::vector<int> vnodes;
       const size_t s0 = plan.w_sten.size();
       std::vector<uint8_t> is_virt;
@@ -208,11 +253,15 @@ bool build_run_plan(const std::vector<LatGeom>& lats, const std::vector<const ui
           const bool s = solid(x, y);
           is_virt.push_back(s);
           if (s) {
-            const auto it = vmap.emplace(y * nx + x, int(vmap.size()));
-            if (it.second) vnodes.push_back(y * nx + x);
-            q.i[a - 1] = uint16_t(it.first->second);
+            const size_t n = size_t(y) * nx + x;
+            if (stamp[n] != int(k)) {
+              stamp[n] = int(k);
+              local[n] = int(vnodes.size());
+              vnodes.push_back(int(n));
+            }
+            q.i[a - 1] = uint16_t(local[n]);
           } else {
-            q.i[a - 1] = uint16_t(slot(x, y));
+            q.i[a - 1] = uint16_t(in_band(x, y));
           }
         }
         plan.w_sten.push_back(q);
@@ -221,19 +270,20 @@ bool build_run_plan(const std::vector<LatGeom>& lats, const std::vector<const ui
         WallSten q{};
         for (int b = 1; b < 9; ++b) {
           const int x = wrap_clamp(node % nx + EXH[b], nx, px), y = wrap_clamp(node / nx + EYH[b], ny, py);
-          q.i[b - 1] = solid(x, y) ? kWallNone : uint16_t(slot(x, y));
+          q.i[b - 1] = solid(x, y) ? kWallNone : uint16_t(in_band(x, y));
         }
         plan.v_sten.push_back(q);
       }
       t.ne = int(extra.size());
+      t.nband = nband;
       for (size_t w = s0; w < plan.w_sten.size(); ++w)
         for (int a = 0; a < 8; ++a)
-          if (is_virt[(w - s0) * 8 + a]) plan.w_sten[w].i[a] = uint16_t(plan.w_sten[w].i[a] + nd + t.ne);
-      t.nw = int(wmap.size());
-      t.nv = int(vmap.size());
+          if (is_virt[(w - s0) * 8 + a]) plan.w_sten[w].i[a] = uint16_t(plan.w_sten[w].i[a] + t.nband);
+      t.nw = nw;
+      t.nv = int(vnodes.size());
       t.ncopy = int(plan.copies.size()) - t.copy0;
       t.nvn = int(plan.vn.size()) - t.vn0;
-      if (nd + t.ne + t.nv >= int(kWallNone) || t.nw >= int(kWallNone)) return false;
+      if (nd + t.ne >= int(kWallNone) || t.nband + t.nv >= int(kWallNone) || t.nw >= int(kWallNone)) return false;
       plan.smem = std::max(plan.smem, run_smem_bytes(t, cs));
       if (plan.smem > max_smem) return false;
     }

@@ -18,17 +18,18 @@ namespace lbcg {
 //   nb     tiles that read what this one writes or write what it reads: those within
 //          kRunReach nodes
 //   extra  the extra slots' nodes (y * nx + x)
+//   band   slots whose rho^N the wall chain reads
 //   w      outermost fluid nodes whose corrected gradient the tile needs: index into the
-//          outermost-fluid list, and the slots of their 8 neighbours (dense, extra, or, after
-//          those, the virtual nodes)
-//   v      virtual (outermost solid) nodes of rho^N: the slots of their fluid neighbours
+//          outermost-fluid list, and where the wall chain has their 8 neighbours (index in band,
+//          or, after those, the virtual nodes)
+//   v      virtual (outermost solid) nodes of rho^N: the indices in band of their fluid neighbours
 //   copy   positions of the n array (tile plus 1 node all round, row-major, (tx + 2) per row)
 //          that hold an outermost fluid node: position, and its index in w
 //   vn     positions that hold an outermost solid node: position, and the indices in w of its
 //          fluid neighbours
 struct RunTile {
   int lat, x0, y0, tx, ty;
-  int nb0, nnb, extra0, ne, w0, nw, v0, nv, copy0, ncopy, vn0, nvn;
+  int nb0, nnb, extra0, ne, band0, nband, w0, nw, v0, nv, copy0, ncopy, vn0, nvn;
   int pad_;
 };
 struct RunVirtN {
@@ -46,11 +47,16 @@ struct RunPlan {
   std::vector<RunTile> tiles;
   std::vector<int> nb, extra, w_ofb;
   std::vector<WallSten> w_sten, v_sten;
+  std::vector<uint16_t> band;
   std::vector<uint32_t> copies;   // position | index in w << 16
   std::vector<RunVirtN> vn;
   size_t smem = 0;                // dynamic shared memory of the largest tile
 };
 
+// Blocks, i.e. tiles, per SM for `cs` bytes per value of the compute type.  FP32 arithmetic: two, so
+// that one works while the other waits for its neighbours.  FP64: one, since the FP64 pipe is
+// the bound and a tile half as large recomputes more of its halo.
+LBCG_HD constexpr int run_blocks(size_t cs) { return cs == 4 ? 2 : 1; }
 // Dynamic shared memory of a tile: `cs` bytes per value of the compute type.
 size_t run_smem_bytes(const RunTile& t, size_t cs);
 

@@ -20,7 +20,10 @@
 // of one pass); on the larger ones instruction issue; in FP64 the FP64 pipe.  Per step, launch per
 // kernel -> resident: 100 x 50 FP64 26.5 -> 12.6 us, 1200 x 80 FP64 72 -> 35.5, FP32 10.5 -> 5.3,
 // 2000 x 102 FP32 17.3 -> 9.4, FP16 18.6 -> 9.3, 8 x 630 x 60 FP32 with Poiseuille inlets 36 -> 12.8
-// (18.4 with the inlet profile evaluated, in FP64, at every read of an edge node).
+// (18.4 with the inlet profile evaluated, in FP64, at every read of an edge node).  FP32 arithmetic:
+// two blocks of 256 threads per SM, whose waits overlap each other's work, against one of 512:
+// 2000 x 102 FP32 9.4 -> 9.1, FP16 9.3 -> 8.7, 8 x 630 x 60 12.8 -> 11.8; with the push offsets of
+// bulk nodes apart from those of wall nodes 8.7, 8.5 and 11.3.
 #include "lbcg_internal.h"
 #include "lbcg_node.cuh"
 
@@ -53,13 +56,12 @@ __device__ __forceinline__ void store_release(unsigned* p, unsigned v) {
 __device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 
 // slot table entry: own index in the low half (0xFFFF: not of the tile), and
-constexpr uint32_t kSlotBand = 1u << 16;     // its rho^N is read by the wall chain
 constexpr uint32_t kSlotEdge = 1u << 17;     // in an open column: Zou-He on every read
 constexpr uint32_t kSlotOutlet = 1u << 18;   // and that column is the outlet
 constexpr int kSlotRow = 20;                 // its row in the table of inlet velocities, from this bit
-// own-node table entry, second word: neighbour-solid mask, and
+// own-node table entry: neighbour-solid mask, column and row in the tile (from bits 16 and 24), and
 constexpr uint32_t kOwnSolid = 1u << 8, kOwnEdge = 1u << 9, kOwnOfb = 1u << 10;
-constexpr uint16_t kNoBulk = 0xFFFF;
+constexpr uint16_t kNone = 0xFFFF;   // no entry (of a position in the bulk, of a slot in the band)
 
 
 template <typename T>
@@ -70,9 +72,9 @@ __device__ __forceinline__ T* carve(unsigned char*& p, size_t n) {
 }
 
 template <typename S, int NT>
-__global__ void __launch_bounds__(NT, 1) k_run(RunArgs A) {
+__global__ void __launch_bounds__(NT, run_blocks(sizeof(typename Store<S>::T))) k_run(RunArgs A) {
   using T = typename Store<S>::T;
-  constexpr int kWallTeam = NT >= 256 ? 128 : 64;   // threads that evaluate a tile's wall nodes beside its bulk nodes
+  constexpr int kWallTeam = 128;   // threads that evaluate a tile's wall nodes beside its bulk nodes
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ LatDev sL;
   const RunTile tl = A.tiles[blockIdx.x];
@@ -82,7 +84,7 @@ __global__ void __launch_bounds__(NT, 1) k_run(RunArgs A) {
   const int ND = CW * (tl.ty + 4), NR = ND + tl.ne, NP = PW * (tl.ty + 2), NO = tl.tx * tl.ty;
   unsigned char* sp = smem;
   T* const srn = carve<T>(sp, NR);             // rho^N of the slots
-  T* const swv = carve<T>(sp, NR + tl.nv);     // the wall chain's rho^N: band slots, then virtual nodes
+  T* const swv = carve<T>(sp, tl.nband + tl.nv);   // the wall chain's rho^N: band slots, then virtual nodes
   T* const snx = carve<T>(sp, NP);             // n and gradient on tile + 1
   T* const sny = carve<T>(sp, NP);
   T* const sgx = carve<T>(sp, NP);
@@ -93,9 +95,10 @@ __global__ void __launch_bounds__(NT, 1) k_run(RunArgs A) {
   T* const sden = carve<T>(sp, tl.nv + tl.nvn);        // Eq. 29 weights of the virtual nodes, of rho^N and of n
   int* const r_off = carve<int>(sp, NR);
   uint32_t* const r_tab = carve<uint32_t>(sp, NR);
+  uint16_t* const r_band = carve<uint16_t>(sp, NR);
   T* const s_u = carve<T>(sp, tl.ty + 8);
   uint16_t* const p_src = carve<uint16_t>(sp, NP);
-  uint2* const o_tab = carve<uint2>(sp, NO);
+  uint32_t* const o_tab = carve<uint32_t>(sp, NO);
   int* const colk = carve<int>(sp, PW);
   int* const rowk = carve<int>(sp, tl.ty + 2);
   WallSten* const w_sten = carve<WallSten>(sp, tl.nw);
@@ -137,6 +140,7 @@ __global__ void __launch_bounds__(NT, 1) k_run(RunArgs A) {
     }
     r_off[i] = solid ? -1 : pop_node(x, y, pitch);
     r_tab[i] = tab;
+    r_band[i] = kNone;
     srn[i] = T(0);
   }
   for (int i = t; i < tl.ty + 8; i += NT) s_u[i] = inlet_u<T>(sL, wrap_or_clamp(tl.y0 - 4 + i, ny, py));
@@ -148,17 +152,15 @@ __global__ void __launch_bounds__(NT, 1) k_run(RunArgs A) {
     const int x = wrap_or_clamp(xr, nx, px), y = wrap_or_clamp(yr, ny, py);
     const int sx = px ? cx : cx + x - xr, sy = py ? cy : cy + y - yr;
     const uint8_t f = fl[(long long)y * pitch + x];
-    p_src[i] = (f & (F_SOLID | F_OFB)) ? kNoBulk : uint16_t((sy + 1) * CW + sx + 1);
+    p_src[i] = (f & (F_SOLID | F_OFB)) ? kNone : uint16_t((sy + 1) * CW + sx + 1);
     snx[i] = sny[i] = sgx[i] = sgy[i] = T(0);
   }
   for (int i = t; i < NO; i += NT) {
     const int lx = i % tl.tx, ly = i / tl.tx;
     const long long k = (long long)(tl.y0 + ly) * pitch + tl.x0 + lx;
     const uint8_t f = fl[k];
-    uint2 e;
-    e.x = uint32_t((ly + 1) * PW + lx + 1) | uint32_t(lx) << 16 | uint32_t(ly) << 24;
-    e.y = uint32_t(nbm[k]) | (f & F_SOLID ? kOwnSolid : 0u) | (f & F_EDGE ? kOwnEdge : 0u) | (f & F_OFB ? kOwnOfb : 0u);
-    o_tab[i] = e;
+    o_tab[i] = uint32_t(nbm[k]) | (f & F_SOLID ? kOwnSolid : 0u) | (f & F_EDGE ? kOwnEdge : 0u) |
+               (f & F_OFB ? kOwnOfb : 0u) | uint32_t(lx) << 16 | uint32_t(ly) << 24;
   }
   for (int i = t; i < PW; i += NT) {
     const int x = wrap_or_clamp(tl.x0 + i - 1, nx, px);
@@ -181,13 +183,7 @@ __global__ void __launch_bounds__(NT, 1) k_run(RunArgs A) {
   }
   for (int i = t; i < tl.ncopy; i += NT) copies[i] = A.copies[tl.copy0 + i];
   __syncthreads();
-  // mark the slots the wall chain reads (several threads may set the same bit)
-  for (int i = t; i < tl.nw + tl.nv; i += NT) {
-    const WallSten q = i < tl.nw ? w_sten[i] : v_sten[i - tl.nw];
-#pragma unroll
-    for (int a = 0; a < 8; ++a)
-      if (q.i[a] < NR) atomicOr(&r_tab[q.i[a]], kSlotBand);
-  }
+  for (int i = t; i < tl.nband; i += NT) r_band[A.band[tl.band0 + i]] = uint16_t(i);
   // the tile's wall nodes have threads of their own beside the bulk nodes' (when it has any)
   const bool walls = tl.nw > 0;
   const int team = walls ? NT - kWallTeam : NT;
@@ -247,14 +243,15 @@ __global__ void __launch_bounds__(NT, 1) k_run(RunArgs A) {
         sf[10 * NO + own] = rhoB;
         sf[11 * NO + own] = irho;
       }
-      if (tab & kSlotBand) swv[i] = rdiv(rsub(rhoR, rhoB), radd(rhoR, rhoB));   // Eq. 12 as k_wall rounds it
+      const uint32_t band = r_band[i];
+      if (band != kNone) swv[band] = rdiv(rsub(rhoR, rhoB), radd(rhoR, rhoB));   // Eq. 12 as k_wall rounds it
     }
     __syncthreads();
     // ---- gradient and n of the bulk nodes of tile + 1, beside the wall chain (Eq. 28-36)
     if (t < team) {
       for (int i = t; i < NP; i += team) {
         const uint32_t c = p_src[i];
-        if (c == kNoBulk) continue;
+        if (c == kNone) continue;
         T ax, ay, nxv, nyv;
         grad_normal<T>(srn + c, CW, eps2, ax, ay, nxv, nyv);
         sgx[i] = ax;
@@ -265,11 +262,12 @@ __global__ void __launch_bounds__(NT, 1) k_run(RunArgs A) {
       if constexpr (sizeof(T) == 8) {
         // what the collision needs of the totals alone, while the wall chain runs
         for (int i = t; i < NO; i += team) {
-          if (o_tab[i].y & kOwnSolid) continue;
+          const uint32_t e = o_tab[i];
+          if (e & kOwnSolid) continue;
           T f[9];
 #pragma unroll
           for (int a = 0; a < 9; ++a) f[a] = sf[a * NO + i];
-          const int c = ((o_tab[i].x >> 24) + 2) * CW + ((o_tab[i].x >> 16) & 0xFFu) + 2;
+          const int c = ((e >> 24) + 2) * CW + ((e >> 16) & 0xFFu) + 2;
           Moments<T> m;
           m.of(f);
           sf[i] = m.e;
@@ -286,7 +284,7 @@ __global__ void __launch_bounds__(NT, 1) k_run(RunArgs A) {
     } else {
       const int w = t - team;
       for (int j = w; j < tl.nv; j += kWallTeam)
-        swv[NR + j] = sL.wetting == 2 ? C.cos_theta : virtual_value<T>(v_sten[j], swv, sden[j]);
+        swv[tl.nband + j] = sL.wetting == 2 ? C.cos_theta : virtual_value<T>(v_sten[j], swv, sden[j]);
       bar_sync(1, kWallTeam);
       for (int j0 = w & ~31; j0 < 2 * tl.nw; j0 += kWallTeam) {   // two lanes per node, whole warps
         const int j = min((j0 + (w & 31)) >> 1, tl.nw - 1), r = w & 1;
@@ -319,9 +317,9 @@ __global__ void __launch_bounds__(NT, 1) k_run(RunArgs A) {
     __syncthreads();
     // ---- curvature, force, collision, recolouring, push
     for (int i = t; i < NO; i += NT) {
-      const uint2 e = o_tab[i];
-      if (e.y & kOwnSolid) continue;
-      const int o1 = e.x & 0xFFFFu, lx = (e.x >> 16) & 0xFFu, ly = e.x >> 24;
+      const uint32_t e = o_tab[i];
+      if (e & kOwnSolid) continue;
+      const int lx = (e >> 16) & 0xFFu, ly = e >> 24, o1 = (ly + 1) * PW + lx + 1;
       const T rhoR = sf[9 * NO + i], rhoB = sf[10 * NO + i], irho = sf[11 * NO + i];
       T f[9], sv;
       Moments<T> m;
@@ -343,8 +341,8 @@ __global__ void __launch_bounds__(NT, 1) k_run(RunArgs A) {
       }
       T dxx, dxy, dyx, dyy;
       grad_n<T>(snx + o1, sny + o1, PW, dxx, dyx, dxy, dyy);
-      const unsigned mask = e.y & 0xFFu;
-      if (sL.wetting == 1 && (e.y & kOwnOfb)) {
+      const unsigned mask = e & 0xFFu;
+      if (sL.wetting == 1 && (e & kOwnOfb)) {
         T nxs[9], nys[9];
 #pragma unroll
         for (int a = 0; a < 9; ++a) {
@@ -364,21 +362,24 @@ __global__ void __launch_bounds__(NT, 1) k_run(RunArgs A) {
       if constexpr (Store<S>::kDeviation) srh = sr_node(srk, kn);
       // streaming (Eq. 15): to x + e_a if that node is fluid; half-way bounce-back into the
       // opposite slot of this node if it is solid; dropped if it lies beyond an open edge
+      int k[9];
+#pragma unroll
+      for (int a = 0; a < 9; ++a) k[a] = rowk[ly + 1 + ey(a)] + colk[lx + 1 + ex(a)] + a * kDir;
+      if (e & (0xFFu | kOwnEdge)) {
+#pragma unroll
+        for (int a = 1; a < 9; ++a) {
+          if (mask & (1u << (a - 1))) k[a] = kn + opp(a) * kDir;
+          const int xr = tl.x0 + lx + ex(a);
+          if ((e & kOwnEdge) && (xr < 0 || xr >= nx)) k[a] = -1;
+        }
+      }
 #pragma unroll
       for (int a = 0; a < 9; ++a) {
-        int k = kn + a * kDir;
-        if (a != 0) {
-          if (e.y & kOwnEdge) {
-            const int xr = tl.x0 + lx + ex(a);
-            if (xr < 0 || xr >= nx) continue;
-          }
-          if (mask & (1u << (a - 1))) k = kn + opp(a) * kDir;
-          else k = rowk[ly + 1 + ey(a)] + colk[lx + 1 + ex(a)] + a * kDir;
-        }
+        if (a != 0 && k[a] < 0) continue;
         T oR, oB;
         rc.out(a, fp, oR, oB);
-        if (checked(in_extent(k, 2, pop_n), A.err))
-          store_pair_sr<S>(dst + k, oR, oB, wgt<T>(a) * C.rho0, sr_bits(srh, a));
+        if (checked(in_extent(k[a], 2, pop_n), A.err))
+          store_pair_sr<S>(dst + k[a], oR, oB, wgt<T>(a) * C.rho0, sr_bits(srh, a));
       }
     }
     __syncthreads();
@@ -391,8 +392,7 @@ __global__ void __launch_bounds__(NT, 1) k_run(RunArgs A) {
 
 __global__ void k_sr_add(uint32_t* epoch, uint32_t n) { *epoch += n; }
 
-template <typename S>
-constexpr int run_threads() { return sizeof(S) == 8 ? 256 : 512; }
+constexpr int kRunThreads = 256;
 
 template <typename S>
 cudaError_t launch(const RunArgs& a, int ntiles, size_t smem, cudaStream_t st) {
@@ -401,19 +401,19 @@ cudaError_t launch(const RunArgs& a, int ntiles, size_t smem, cudaStream_t st) {
   at[0].val.cooperative = 1;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(unsigned(ntiles));
-  cfg.blockDim = dim3(run_threads<S>());
+  cfg.blockDim = dim3(kRunThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_run<S, run_threads<S>()>, a);
+  return cudaLaunchKernelEx(&cfg, k_run<S, kRunThreads>, a);
 }
 
 template <typename S>
 cudaError_t prepare(size_t smem, int* per_sm) {
-  cudaError_t e = cudaFuncSetAttribute(k_run<S, run_threads<S>()>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  cudaError_t e = cudaFuncSetAttribute(k_run<S, kRunThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
   if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_run<S, run_threads<S>()>, run_threads<S>(), smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_run<S, kRunThreads>, kRunThreads, smem);
   return e;
 }
 

@@ -117,19 +117,22 @@ static void check(const std::vector<Box>& boxes, int max_tiles, size_t cs) {
       require(e.lat == t.lat, "outermost fluid node of the same lattice");
       return e.y * b.nx + e.x;
     };
+    std::set<int> band(plan.band.begin() + t.band0, plan.band.begin() + t.band0 + t.nband);
+    require(int(band.size()) == t.nband && (band.empty() || *band.rbegin() < nr), "band slots");
     std::vector<int> virt(t.nv, -1);
     for (int w = 0; w < t.nw; ++w) {
       const int n = of_w(w);
       for (int a = 1; a < 9; ++a) {
         const int m = node(n % b.nx + EXH[a], n / b.nx + EYH[a]);
         const int i = plan.w_sten[t.w0 + w].i[a - 1];
-        require(i < nr + t.nv, "stencil index");
+        require(i < t.nband + t.nv, "stencil index");
         if (b.solid[m]) {
-          require(i >= nr, "a solid neighbour is a virtual node");
-          require(virt[i - nr] == -1 || virt[i - nr] == m, "one virtual node per index");
-          virt[i - nr] = m;
+          const int j = i - t.nband;
+          require(j >= 0, "a solid neighbour is a virtual node");
+          require(virt[j] == -1 || virt[j] == m, "one virtual node per index");
+          virt[j] = m;
         } else {
-          require(i < nr && at[i] == m, "a fluid neighbour's slot");
+          require(i < t.nband && at[plan.band[t.band0 + i]] == m, "a fluid neighbour's slot");
         }
       }
     }
@@ -138,7 +141,8 @@ static void check(const std::vector<Box>& boxes, int max_tiles, size_t cs) {
       for (int a = 1; a < 9; ++a) {
         const int m = node(virt[v] % b.nx + EXH[a], virt[v] / b.nx + EYH[a]);
         const int i = plan.v_sten[t.v0 + v].i[a - 1];
-        require(b.solid[m] ? i == kWallNone : (i < nr && at[i] == m), "a virtual node's neighbours");
+        require(b.solid[m] ? i == kWallNone : (i < t.nband && at[plan.band[t.band0 + i]] == m),
+                "a virtual node's neighbours");
       }
     }
     const int pw = t.tx + 2, np = pw * (t.ty + 2);
