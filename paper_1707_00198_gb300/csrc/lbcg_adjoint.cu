@@ -59,44 +59,44 @@ template <typename R>
 __device__ __forceinline__ int mapy(const AdjDevT<R>& A, int v) { return wrap_or_clamp(v, A.L.ny, A.L.bcy == BC_PERIODIC); }
 
 // ------------------------------------------------------------------ forward intermediates
-template <typename R>
-__device__ __forceinline__ void fwd_local_body(const AdjDevT<R>& A, const int i) {
+template <typename R, bool kGather>
+__device__ __forceinline__ void fwd_local_body(const AdjDevT<R>& A, const void* src, const int i, const int p) {
   const int x = i % A.L.nx, y = i / A.L.nx;
-  const int N = A.N;
+  const int M = A.M;
   // The kernels of the reverse sweep run a few warps per SM, so each memory round trip on a
   // thread's path counts: a node's loads are issued together, before its solid test (the
   // slots of a solid node are read but not used).
   const bool solid = is_solid(A, x, y);
-  A.lnt_x[i] = A.lnt_y[i] = A.lrnt[i] = R(0.0);
+  if constexpr (!kGather) A.lnt_x[i] = A.lnt_y[i] = A.lrnt[i] = R(0.0);
   R fr[9], fb[9], rR, rB;
   if (A.src_fp32) {
     // FP32 forward: its post-Zou-He populations, converted to the reverse arithmetic
     float fr32[9], fb32[9];
-    load_node<float>(A.L, static_cast<const float*>(A.src), x, y, fr32, fb32);
+    load_node<float>(A.L, static_cast<const float*>(src), x, y, fr32, fb32);
     for (int a = 0; a < 9; ++a) {
       fr[a] = R(fr32[a]);
       fb[a] = R(fb32[a]);
     }
   } else {
     double fr64[9], fb64[9];
-    load_node<double>(A.L, static_cast<const double*>(A.src), x, y, fr64, fb64);
+    load_node<double>(A.L, static_cast<const double*>(src), x, y, fr64, fb64);
     for (int a = 0; a < 9; ++a) {
       fr[a] = R(fr64[a]);
       fb[a] = R(fb64[a]);
     }
   }
   if (solid) {
-    for (int a = 0; a < 9; ++a) A.fr[a * N + i] = A.fb[a * N + i] = R(0.0);
-    A.rr[i] = A.rb[i] = A.rn[i] = R(0.0);
+    for (int a = 0; a < 9; ++a) A.fr[a * M + p] = A.fb[a * M + p] = R(0.0);
+    A.rr[p] = A.rb[p] = A.rn[i] = R(0.0);
     return;
   }
   for (int a = 0; a < 9; ++a) {
-    A.fr[a * N + i] = fr[a];
-    A.fb[a * N + i] = fb[a];
+    A.fr[a * M + p] = fr[a];
+    A.fb[a * M + p] = fb[a];
   }
   A.rn[i] = colour_indicator(fr, fb, rR, rB);
-  A.rr[i] = rR;
-  A.rb[i] = rB;
+  A.rr[p] = rR;
+  A.rb[p] = rB;
 }
 
 // Sum of the D2Q9 weights toward the fluid neighbours of a solid node (Eq. 29 denominator)
@@ -150,22 +150,21 @@ __device__ void scatter_field(const AdjDevT<R>& A, R* acc0, R* acc1, int x, int 
   }
 }
 
-template <typename R>
-__device__ __forceinline__ void fwd_grad_body(const AdjDevT<R>& A, const int i) {
-  const int x = i % A.L.nx, y = i / A.L.nx;
-  const uint8_t f = flag_at(A, x, y);
-  const unsigned msk = A.nbm[i];
+// field(a): rho^N (of Eq. 28-29's reading) at the neighbour in direction a
+template <typename R, typename F>
+__device__ __forceinline__ void fwd_grad_body(const AdjDevT<R>& A, const int i, const int p, const uint8_t f, F field) {
   const R nsx = A.nsx[i], nsy = A.nsy[i];
   const R c = A.cos_t[i], s = A.sin_t[i];
-  A.pick[i] = 0;
+  A.pick[p] = 0;
   if (f & F_SOLID) {
-    A.grx[i] = A.gry[i] = A.gcx[i] = A.gcy[i] = R(0.0);
+    A.grx[p] = A.gry[p] = A.gcx[p] = A.gcy[p] = R(0.0);
     A.nxv[i] = A.nyv[i] = R(0.0);
     return;
   }
   R gx = R(0.0), gy = R(0.0);
+#pragma unroll
   for (int a = 1; a < 9; ++a) {
-    const R t = rmul(wgt<R>(a), read_field(A, A.rn, mapx(A, x + ex(a)), mapy(A, y + ey(a)), mask_bit(msk, a)));
+    const R t = rmul(wgt<R>(a), field(a));
     if (ex(a) == 1) gx = radd(gx, t);
     if (ex(a) == -1) gx = radd(gx, -t);
     if (ey(a) == 1) gy = radd(gy, t);
@@ -173,10 +172,10 @@ __device__ __forceinline__ void fwd_grad_body(const AdjDevT<R>& A, const int i) 
   }
   gx = rdiv(gx, R(1.0 / 3.0));
   gy = rdiv(gy, R(1.0 / 3.0));
-  A.grx[i] = gx;
-  A.gry[i] = gy;
+  A.grx[p] = gx;
+  A.gry[p] = gy;
   R cgx = gx, cgy = gy;
-  const R eps = R(A.L.grad_eps);
+  const R eps = A.C.grad_eps;
   const R mag = rsqrt_(radd(rmul(gx, gx), rmul(gy, gy)));
   if ((f & F_OFB) && mag > eps) {
     const R esx = rdiv(gx, mag), esy = rdiv(gy, mag);
@@ -186,65 +185,82 @@ __device__ __forceinline__ void fwd_grad_body(const AdjDevT<R>& A, const int i) 
     const R d1 = rsqrt_(radd(rmul(a1, a1), rmul(b1, b1)));
     const R d2 = rsqrt_(radd(rmul(a2, a2), rmul(b2, b2)));
     const bool one = d1 <= d2;
-    A.pick[i] = one ? 1 : 2;
+    A.pick[p] = one ? 1 : 2;
     cgx = rmul(mag, one ? f1x : f2x);
     cgy = rmul(mag, one ? f1y : f2y);
   }
-  A.gcx[i] = cgx;
-  A.gcy[i] = cgy;
+  A.gcx[p] = cgx;
+  A.gcy[p] = cgy;
   const R m2 = sqrt(cgx * cgx + cgy * cgy);
   A.nxv[i] = m2 > eps ? cgx / m2 : R(0.0);
   A.nyv[i] = m2 > eps ? cgy / m2 : R(0.0);
 }
 
 template <typename R>
-__device__ __forceinline__ void fwd_dn_body(const AdjDevT<R>& A, const int i) {
+__device__ __forceinline__ void fwd_grad_node(const AdjDevT<R>& A, const int i) {
   const int x = i % A.L.nx, y = i / A.L.nx;
-  const int N = A.N;
-  R d[4] = {0, 0, 0, 0};
-  const bool solid = is_solid(A, x, y);
   const unsigned msk = A.nbm[i];
+  fwd_grad_body(A, i, i, flag_at(A, x, y), [&](int a) {
+    return read_field(A, A.rn, mapx(A, x + ex(a)), mapy(A, y + ey(a)), mask_bit(msk, a));
+  });
+}
+
+// fx(a), fy(a): n_x and n_y at the neighbour in direction a
+template <typename R, typename F, typename G>
+__device__ __forceinline__ void fwd_dn_body(const AdjDevT<R>& A, const int p, const bool solid, F fx, G fy) {
+  const int M = A.M;
+  R d[4] = {0, 0, 0, 0};
   if (!solid) {
+#pragma unroll
     for (int a = 1; a < 9; ++a) {
-      const int x2 = mapx(A, x + ex(a)), y2 = mapy(A, y + ey(a));
-      const bool sn = mask_bit(msk, a);
-      const R tx = wgt<R>(a) * read_field(A, A.nxv, x2, y2, sn);
-      const R ty = wgt<R>(a) * read_field(A, A.nyv, x2, y2, sn);
+      const R tx = wgt<R>(a) * fx(a);
+      const R ty = wgt<R>(a) * fy(a);
       d[0] += ex(a) * tx;
       d[1] += ey(a) * tx;
       d[2] += ex(a) * ty;
       d[3] += ey(a) * ty;
     }
   }
-  for (int q = 0; q < 4; ++q) A.dn[q * N + i] = R(3.0) * d[q];
+  for (int q = 0; q < 4; ++q) A.dn[q * M + p] = R(3.0) * d[q];
+}
+template <typename R>
+__device__ __forceinline__ void fwd_dn_node(const AdjDevT<R>& A, const int i) {
+  const int x = i % A.L.nx, y = i / A.L.nx;
+  const unsigned msk = A.nbm[i];
+  auto at = [&](const R* v, int a) {
+    return read_field(A, v, mapx(A, x + ex(a)), mapy(A, y + ey(a)), mask_bit(msk, a));
+  };
+  fwd_dn_body(A, i, is_solid(A, x, y), [&](int a) { return at(A.nxv, a); }, [&](int a) { return at(A.nyv, a); });
 }
 
 // ------------------------------------------------------------------ reverse kernels
 // Transpose of the push (Eq. 15, half-way bounce-back, open edges) and the reverse of the
 // node-local part of the step.
-template <typename R>
-__device__ __forceinline__ void adj_collide_body(const AdjDevT<R>& A, const int i) {
+// kGather: instead of scattering the transpose of grad n, the adjoints of d_x n_x, d_y n_x (= that
+// of d_x n_y) and d_y n_y are stored, and the nodes that were read gather them (k_reverse).
+template <typename R, bool kGather>
+__device__ __forceinline__ void adj_collide_body(const AdjDevT<R>& A, const R* lam_next, const int i, const int p,
+                                                 const bool solid, const unsigned msk, R& d_sigma, R& d_hR, R& d_hB,
+                                                 R* src0 = nullptr, R* src1 = nullptr, R* src2 = nullptr) {
   const int x = i % A.L.nx, y = i / A.L.nx;
-  const int N = A.N;
+  const int N = A.N, M = A.M;
+  d_sigma = d_hR = d_hB = R(0.0);
   const LatDev& L = A.L;
-  // the node's masks, forward intermediates and parameter adjoints so far, all in flight
-  // together before the solid test
-  const bool solid = is_solid(A, x, y);
-  const unsigned msk = A.nbm[i];
+  const LatConst<R>& C = A.C;
+  // the node's forward intermediates, all in flight together before the solid test
   R fr[9], fb[9], f[9];
   for (int a = 0; a < 9; ++a) {
-    fr[a] = A.fr[a * N + i];
-    fb[a] = A.fb[a * N + i];
+    fr[a] = A.fr[a * M + p];
+    fb[a] = A.fb[a * M + p];
     f[a] = fr[a] + fb[a];
   }
-  const R rhoR = A.rr[i], rhoB = A.rb[i], rn = A.rn[i];
+  const R rhoR = A.rr[p], rhoB = A.rb[p], rn = A.rn[i];
   const R nxo = A.nxv[i], nyo = A.nyv[i];
-  const R gx = A.gcx[i], gy = A.gcy[i];
-  const R dxx = A.dn[i], dxy = A.dn[N + i], dyx = A.dn[2 * N + i], dyy = A.dn[3 * N + i];
-  const double p_hR0 = A.p_hR[i], p_hB0 = A.p_hB[i], p_sigma0 = A.p_sigma[i];
+  const R gx = A.gcx[p], gy = A.gcy[p];
+  const R dxx = A.dn[p], dxy = A.dn[M + p], dyx = A.dn[2 * M + p], dyy = A.dn[3 * M + p];
   if (solid) {
-    for (int a = 0; a < 9; ++a) A.lf_r[a * N + i] = A.lf_b[a * N + i] = R(0.0);
-    A.ln_x[i] = A.ln_y[i] = A.lg_x[i] = A.lg_y[i] = A.lrn[i] = R(0.0);
+    for (int a = 0; a < 9; ++a) A.lf_r[a * M + p] = A.lf_b[a * M + p] = R(0.0);
+    A.ln_x[p] = A.ln_y[p] = A.lg_x[p] = A.lg_y[p] = A.lrn[p] = R(0.0);
     return;
   }
   const bool px = L.bcx == BC_PERIODIC, py = L.bcy == BC_PERIODIC;
@@ -260,21 +276,21 @@ __device__ __forceinline__ void adj_collide_body(const AdjDevT<R>& A, const int 
       if (mask_bit(msk, a)) slot = opp(a);
       else j = yd * L.nx + xd;
     }
-    mR[a] = A.lam_next[(2 * slot) * N + j];
-    mB[a] = A.lam_next[(2 * slot + 1) * N + j];
+    mR[a] = lam_next[(2 * slot) * N + j];
+    mB[a] = lam_next[(2 * slot + 1) * N + j];
   }
   // forward recomputation of the node-local quantities
   const R rho = rhoR + rhoB, ir = R(1.0) / rho;
   const R kappa = -nxo * nxo * dyy - nyo * nyo * dxx + nxo * nyo * (dxy + dyx);
-  const R hsk = R(0.5) * R(L.sigma) * kappa;
+  const R hsk = R(0.5) * C.sigma * kappa;
   const R Fx = hsk * gx, Fy = hsk * gy;
   const R jx = f[1] - f[3] + f[5] - f[6] - f[7] + f[8];
   const R jy = f[2] - f[4] + f[5] + f[6] - f[7] - f[8];
   const R ux = (jx + R(0.5) * Fx) * ir, uy = (jy + R(0.5) * Fy) * ir;
-  const R inv_nu = (1 + rn) * R(L.h_inv_nuR) + (1 - rn) * R(L.h_inv_nuB);
+  const R inv_nu = (1 + rn) * C.h_inv_nuR + (1 - rn) * C.h_inv_nuB;
   const R den_sv = R(3.0) + R(0.5) * inv_nu;
   const R sv = inv_nu / den_sv;
-  const R se = L.s_e, seps = L.s_eps, sq = L.s_q, beta = L.beta;
+  const R se = C.s_e, seps = C.s_eps, sq = C.s_q, beta = C.beta;
   const R s14 = f[1] + f[2] + f[3] + f[4], s58 = f[5] + f[6] + f[7] + f[8];
   const R me = -4 * f[0] - s14 + 2 * s58;
   const R meps = 4 * f[0] - 2 * s14 + s58;
@@ -391,9 +407,9 @@ __device__ __forceinline__ void adj_collide_body(const AdjDevT<R>& A, const int 
   }
   // sv = inv_nu / (3 + inv_nu / 2); inv_nu = (1 + rn) hR + (1 - rn) hB
   const R linv = lsv * R(3.0) / (den_sv * den_sv);
-  R lrn_loc = (R(L.h_inv_nuR) - R(L.h_inv_nuB)) * linv;
-  A.p_hR[i] = p_hR0 + (1 + rn) * linv;
-  A.p_hB[i] = p_hB0 + (1 - rn) * linv;
+  R lrn_loc = (C.h_inv_nuR - C.h_inv_nuB) * linv;
+  d_hR = (1 + rn) * linv;
+  d_hB = (1 - rn) * linv;
   // u = (j + F/2) / rho
   const R ljx = lux * ir, ljy = luy * ir;
   lFx += R(0.5) * ljx;
@@ -403,13 +419,17 @@ __device__ __forceinline__ void adj_collide_body(const AdjDevT<R>& A, const int 
   // F = (sigma kappa / 2) g
   const R lhsk = gx * lFx + gy * lFy;
   const R lgx = hsk * lFx, lgy = hsk * lFy;
-  A.p_sigma[i] = p_sigma0 + R(0.5) * kappa * lhsk;
-  const R lk = R(0.5) * R(L.sigma) * lhsk;
+  d_sigma = R(0.5) * kappa * lhsk;
+  const R lk = R(0.5) * C.sigma * lhsk;
   // kappa = -nx^2 dyy - ny^2 dxx + nx ny (dxy + dyx)
   lnx += (-2 * nxo * dyy + nyo * (dxy + dyx)) * lk;
   lny += (-2 * nyo * dxx + nxo * (dxy + dyx)) * lk;
   // transpose of grad n = 3 sum_a w_a e_a n~(x + e_a) (Eq. 28 on the Eq. 29-filled n)
-  if (lk != R(0.0)) {
+  if constexpr (kGather) {
+    src0[i] = -nyo * nyo * lk;
+    src1[i] = nxo * nyo * lk;
+    src2[i] = -nxo * nxo * lk;
+  } else if (lk != R(0.0)) {
     const R lxx = -nyo * nyo * lk;   // adjoint of d_x n_x
     const R lxy = nxo * nyo * lk;    // d_y n_x
     const R lyx = nxo * nyo * lk;    // d_x n_y
@@ -425,33 +445,44 @@ __device__ __forceinline__ void adj_collide_body(const AdjDevT<R>& A, const int 
   lrhoR += lrho;
   lrhoB += lrho;
   for (int a = 0; a < 9; ++a) {
-    A.lf_r[a * N + i] = lf[a] + lrhoR;
-    A.lf_b[a * N + i] = lf[a] + lrhoB;
+    A.lf_r[a * M + p] = lf[a] + lrhoR;
+    A.lf_b[a * M + p] = lf[a] + lrhoB;
   }
-  A.lrn[i] = lrn_loc;
-  A.ln_x[i] = lnx;
-  A.ln_y[i] = lny;
-  A.lg_x[i] = lgx;
-  A.lg_y[i] = lgy;
+  A.lrn[p] = lrn_loc;
+  A.ln_x[p] = lnx;
+  A.ln_y[p] = lny;
+  A.lg_x[p] = lgx;
+  A.lg_y[p] = lgy;
+}
+
+// d_sigma, d_hR, d_hB: this step's share of the parameter adjoints
+template <typename R>
+__device__ __forceinline__ void adj_collide_node(const AdjDevT<R>& A, const int i) {
+  const double p_hR0 = A.p_hR[i], p_hB0 = A.p_hB[i], p_sigma0 = A.p_sigma[i];
+  R ds, dR, dB;
+  adj_collide_body<R, false>(A, A.lam_next, i, i, A.sol[i] != 0, A.nbm[i], ds, dR, dB);
+  A.p_sigma[i] = p_sigma0 + ds;
+  A.p_hR[i] = p_hR0 + dR;
+  A.p_hB[i] = p_hB0 + dB;
 }
 
 // Reverse of n = g_c / |g_c| (zero below the guard), of Eq. 30-36 (g_c = |g_r| n_f(theta) on
 // Omega_Fb, g_c = g_r elsewhere), and the transpose of the raw gradient (Eq. 28 on the
 // Eq. 29-filled rho^N), scattered onto rho^N.
+// lntx, lnty: the adjoint of n through the neighbours' grad n.  Returns in lrx, lry the adjoint of
+// the raw gradient (zero on a solid node), in d_theta this step's share of dJ/d theta.
 template <typename R>
-__device__ __forceinline__ void adj_normal_body(const AdjDevT<R>& A, const int i) {
-  const int x = i % A.L.nx, y = i / A.L.nx;
+__device__ __forceinline__ void adj_normal_body(const AdjDevT<R>& A, const int i, const int p, const bool solid, R lntx,
+                                                R lnty, R& lrx, R& lry, R& d_theta) {
   // everything the node reads, in flight together before the solid test
-  const bool solid = is_solid(A, x, y);
-  const unsigned msk = A.nbm[i];
-  const R lnx = A.ln_x[i] + A.lnt_x[i], lny = A.ln_y[i] + A.lnt_y[i];
-  R lgx = A.lg_x[i], lgy = A.lg_y[i];
-  const R gcx = A.gcx[i], gcy = A.gcy[i];
-  const int pick = A.pick[i];
-  const R grx = A.grx[i], gry = A.gry[i];
+  const R lnx = A.ln_x[p] + lntx, lny = A.ln_y[p] + lnty;
+  R lgx = A.lg_x[p], lgy = A.lg_y[p];
+  const R gcx = A.gcx[p], gcy = A.gcy[p];
+  const int pick = A.pick[p];
+  const R grx = A.grx[p], gry = A.gry[p];
   const R nsx = A.nsx[i], nsy = A.nsy[i];
   const R c = A.cos_t[i], s = A.sin_t[i];
-  const double p_theta0 = A.p_theta[i];
+  lrx = lry = d_theta = R(0.0);
   if (solid) return;
   {
     const R gx = gcx, gy = gcy;
@@ -463,7 +494,8 @@ __device__ __forceinline__ void adj_normal_body(const AdjDevT<R>& A, const int i
       lgy += (lny - ny * dot) * im;
     }
   }
-  R lrx = lgx, lry = lgy;
+  lrx = lgx;
+  lry = lgy;
   if (pick != 0) {
     const R gx = grx, gy = gry;
     const R m = sqrt(gx * gx + gy * gy);
@@ -482,8 +514,17 @@ __device__ __forceinline__ void adj_normal_body(const AdjDevT<R>& A, const int i
     const R proj = (nfx * lgx + nfy * lgy) / m;
     lrx = gx * proj;
     lry = gy * proj;
-    A.p_theta[i] = p_theta0 + m * (dfx * lgx + dfy * lgy);
+    d_theta = m * (dfx * lgx + dfy * lgy);
   }
+}
+template <typename R>
+__device__ __forceinline__ void adj_normal_node(const AdjDevT<R>& A, const int i) {
+  const int x = i % A.L.nx, y = i / A.L.nx;
+  const unsigned msk = A.nbm[i];
+  const double p_theta0 = A.p_theta[i];
+  R lrx, lry, dt;
+  adj_normal_body(A, i, i, is_solid(A, x, y), A.lnt_x[i], A.lnt_y[i], lrx, lry, dt);
+  if (dt != R(0.0)) A.p_theta[i] = p_theta0 + dt;
   if (lrx != R(0.0) || lry != R(0.0))
     for (int a = 1; a < 9; ++a)
       scatter_field(A, A.lrnt, static_cast<R*>(nullptr), mapx(A, x + ex(a)), mapy(A, y + ey(a)), mask_bit(msk, a),
@@ -492,20 +533,19 @@ __device__ __forceinline__ void adj_normal_body(const AdjDevT<R>& A, const int i
 
 // reverse of rho^N = (rhoR - rhoB)/(rhoR + rhoB) and of the Zou-He columns
 template <typename R>
-__device__ __forceinline__ void adj_rho_body(const AdjDevT<R>& A, const int i) {
+__device__ __forceinline__ void adj_rho_body(const AdjDevT<R>& A, R* lam, const int i, const int p, const bool solid, R lrnt) {
   const int x = i % A.L.nx, y = i / A.L.nx;
-  const int N = A.N;
+  const int N = A.N, M = A.M;
   // the node's inputs, in flight together before the solid test
-  const bool solid = is_solid(A, x, y);
-  const R lrn = A.lrn[i] + A.lrnt[i];
-  const R rR = A.rr[i], rB = A.rb[i];
+  const R lrn = A.lrn[p] + lrnt;
+  const R rR = A.rr[p], rB = A.rb[p];
   R lr[9], lb[9];
   for (int a = 0; a < 9; ++a) {
-    lr[a] = A.lf_r[a * N + i];
-    lb[a] = A.lf_b[a * N + i];
+    lr[a] = A.lf_r[a * M + p];
+    lb[a] = A.lf_b[a * M + p];
   }
   if (solid) {
-    for (int a = 0; a < 18; ++a) A.lam[a * N + i] = R(0.0);
+    for (int a = 0; a < 18; ++a) lam[a * N + i] = R(0.0);
     return;
   }
   const R rho = rR + rB;
@@ -541,8 +581,8 @@ __device__ __forceinline__ void adj_rho_body(const AdjDevT<R>& A, const int i) {
     const int known[6] = {0, 1, 2, 4, 5, 8};
     R kR = 0, kT = 0;
     for (int q = 0; q < 6; ++q) {
-      kR += FR[known[q] * N + i];
-      kT += FR[known[q] * N + i] + FB[known[q] * N + i];
+      kR += FR[known[q] * M + p];
+      kT += FR[known[q] * M + p] + FB[known[q] * M + p];
     }
     const R frac = kT != 0 ? kR / kT : R(0.0);
     R lt[9], lfrac = 0;
@@ -550,7 +590,7 @@ __device__ __forceinline__ void adj_rho_body(const AdjDevT<R>& A, const int i) {
     const int unk[3] = {3, 6, 7};
     for (int q = 0; q < 3; ++q) {
       const int uu = unk[q];
-      const R fu = FR[uu * N + i] + FB[uu * N + i];
+      const R fu = FR[uu * M + p] + FB[uu * M + p];
       lt[uu] = frac * lr[uu] + (1 - frac) * lb[uu];   // adjoint of the total f_u
       lfrac += fu * (lr[uu] - lb[uu]);
     }
@@ -580,8 +620,8 @@ __device__ __forceinline__ void adj_rho_body(const AdjDevT<R>& A, const int i) {
     }
   }
   for (int a = 0; a < 9; ++a) {
-    A.lam[(2 * a) * N + i] = sr[a];
-    A.lam[(2 * a + 1) * N + i] = sb[a];
+    lam[(2 * a) * N + i] = sr[a];
+    lam[(2 * a + 1) * N + i] = sb[a];
   }
 }
 
@@ -614,20 +654,20 @@ cudaError_t launch_dep(void (*k)(P...), int grid, cudaStream_t st, Q... args) {
 template <typename R>
 __global__ void __launch_bounds__(kAdjThreads) k_fwd_local(AdjDevT<R> A) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < A.N) fwd_local_body(A, i);
+  if (i < A.N) (fwd_local_body<R, false>(A, A.src, i, i));
 }
 template <typename R>
 __global__ void __launch_bounds__(kAdjThreads) k_fwd_grad(AdjDevT<R> A) {
   dep_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < A.N) fwd_grad_body(A, i);
+  if (i < A.N) fwd_grad_node(A, i);
   dep_trigger();
 }
 template <typename R>
 __global__ void __launch_bounds__(kAdjThreads) k_fwd_dn(AdjDevT<R> A) {
   dep_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < A.N) fwd_dn_body(A, i);
+  if (i < A.N) fwd_dn_node(A, i);
   dep_trigger();
 }
 
@@ -644,8 +684,8 @@ __global__ void __launch_bounds__(kAdjThreads) k_rev_collide(AdjDevT<R> A, AdjDe
   const int i = (rev ? blockIdx.x : blockIdx.x - nrev) * blockDim.x + threadIdx.x;
   dep_wait();
   if (i < A.N) {
-    if (rev) adj_collide_body(A, i);
-    else fwd_local_body(B, i);
+    if (rev) adj_collide_node(A, i);
+    else (fwd_local_body<R, false>(B, B.src, i, i));
   }
   dep_trigger();
 }
@@ -655,8 +695,8 @@ __global__ void __launch_bounds__(kAdjThreads) k_rev_normal(AdjDevT<R> A, AdjDev
   const int i = (rev ? blockIdx.x : blockIdx.x - nrev) * blockDim.x + threadIdx.x;
   dep_wait();
   if (i < A.N) {
-    if (rev) adj_normal_body(A, i);
-    else fwd_grad_body(B, i);
+    if (rev) adj_normal_node(A, i);
+    else fwd_grad_node(B, i);
   }
   dep_trigger();
 }
@@ -666,15 +706,326 @@ __global__ void __launch_bounds__(kAdjThreads) k_rev_rho(AdjDevT<R> A, AdjDevT<R
   const int i = (rev ? blockIdx.x : blockIdx.x - nrev) * blockDim.x + threadIdx.x;
   dep_wait();
   if (i < A.N) {
-    if (rev) adj_rho_body(A, i);
-    else fwd_dn_body(B, i);
+    if (rev) adj_rho_body(A, A.lam, i, i, A.sol[i] != 0, A.lrnt[i]);
+    else fwd_dn_node(B, i);
   }
   dep_trigger();
 }
 template <typename R>
 __global__ void __launch_bounds__(kAdjThreads) k_adj_rho(AdjDevT<R> A) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < A.N) adj_rho_body(A, i);
+  if (i < A.N) adj_rho_body(A, A.lam, i, i, A.sol[i] != 0, A.lrnt[i]);
+}
+
+// ------------------------------------------------------------------ resident reverse sweep
+// A checkpoint segment's whole reverse sweep in one cooperative launch, on lattices that the
+// resident step kernel holds: one block per tile of its plan, a thread per node for the reverse
+// stages and, in warps of their own beside them, a thread per node for the forward intermediates.
+// The stages reach at most two nodes beyond a node, so between two stages a block waits only for
+// the tiles around it (the plan's neighbours, a flag per tile), as the step kernel does.
+//
+// Where the launched stages scatter with atomics and evaluate Eq. 29 on the fly (chains of
+// dependent loads on every node next to a wall, which set the pace of the whole lattice: up to
+// 20,000 cycles a stage), the tile plus two nodes all round is brought into shared memory in one
+// round of loads: the virtual values of its solid nodes are filled in once for all readers, and
+// the transposes are gathers (a node from the nodes that read it, a solid node likewise, its fluid
+// neighbours their shares of it).  What only a node's own two threads use stays in shared memory.
+// 400 x 42, FP32 forward and reverse, us per step of the whole gradient (800 steps): launched
+// stages 33.8 (with the resident forward steps), resident with the launched stages' bodies 44.7,
+// with tiles in shared memory 26.1, with the node's own values there too 24.0, beside the
+// recompute 22.0; FP64 reverse of an FP32 forward 85 -> 57, FP64 both 124 -> 89.  What bounds it: three
+// waits per reverse step (about 4,000 cycles each with the fence before them) and the latency of
+// the stages (6,100, 5,300 and 4,100 cycles for one or two warps per scheduler).
+__device__ __forceinline__ unsigned flag_acquire(const unsigned* p) {
+  unsigned v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void flag_release(unsigned* p, unsigned v) {
+  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+__device__ __forceinline__ void half_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+
+// (FP32: held to 128 registers, so that two blocks of 128 threads fit on an SM beside two of the
+// step kernel's that recompute the next segment: 24.0 -> 22.0 us per step on 400 x 42.)
+template <typename R>
+__global__ void __launch_bounds__(kRevMaxThreads, sizeof(R) == 4 ? 2 : 1) k_reverse(const __grid_constant__ RevRunT<R> P) {
+  __shared__ int s_node[kRevMaxSlots];         // node of each slot of tile + 2 (wrapped or clamped)
+  __shared__ uint8_t s_mask[kRevMaxSlots];     // its neighbour-solid mask
+  __shared__ uint8_t s_kind[kRevMaxSlots];     // bit 0: solid, bit 1: beyond an open or closed edge
+  __shared__ uint16_t s_list[kRevMaxSlots];    // solid slots of tile + 1
+  __shared__ uint16_t s_ref[kRevMaxSlots];     // and the slot of the node each stands for
+  __shared__ R s_den[kRevMaxSlots];            // and its Eq. 29 weight
+  __shared__ R s_f[2][kRevMaxSlots];           // forward: the field of the stage (two components)
+  __shared__ R s_q[3][kRevMaxSlots];           // reverse: what the stage gathers
+  __shared__ R s_acc[2][kRevMaxSlots];         // reverse: a solid node's adjoint over its weight
+  __shared__ int s_nlist;
+  __shared__ AdjDevT<R> s_V[2];
+  // what only the node's own threads use, in shared memory (dynamic): the two sets of forward
+  // intermediates and the reverse arrays, M values each
+  extern __shared__ __align__(16) unsigned char s_own[];
+  const RunTile tl = P.tiles[blockIdx.x];
+  const LatDev& L = P.V[0].L;
+  const int nx = L.nx, ny = L.ny;
+  const bool px = L.bcx == BC_PERIODIC, py = L.bcy == BC_PERIODIC, inout = L.bcx == BC_INOUT;
+  const int half = blockDim.x / 2, u = threadIdx.x < half ? threadIdx.x : threadIdx.x - half;
+  const bool rev = threadIdx.x < half;   // whole warps
+  const bool mine = u < tl.tx * tl.ty;
+  const int lx = u % tl.tx, ly = u / tl.tx, x = tl.x0 + lx, y = tl.y0 + ly;
+  const int i = y * nx + x;
+  const int CW = tl.tx + 4, CH = tl.ty + 4, ns = CW * CH;
+  const int c = (ly + 2) * CW + lx + 2;   // this node's slot
+  const int M = half;
+  if (threadIdx.x == 0) {
+    s_nlist = 0;
+    R* w = reinterpret_cast<R*>(s_own);
+    auto take = [&](int n) {
+      R* r = w;
+      w += n * M;
+      return r;
+    };
+    for (int q = 0; q < 2; ++q) {
+      AdjDevT<R>& V = s_V[q];
+      V = P.V[q];
+      V.M = M;
+      V.fr = take(9);
+      V.fb = take(9);
+      V.rr = take(1);
+      V.rb = take(1);
+      V.grx = take(1);
+      V.gry = take(1);
+      V.gcx = take(1);
+      V.gcy = take(1);
+      V.dn = take(4);
+    }
+    R* const lf_r = take(9);
+    R* const lf_b = take(9);
+    R* const lr = take(5);
+    int* const pick = reinterpret_cast<int*>(w);
+    for (int q = 0; q < 2; ++q) {
+      AdjDevT<R>& V = s_V[q];
+      V.lf_r = lf_r;
+      V.lf_b = lf_b;
+      V.ln_x = lr;
+      V.ln_y = lr + M;
+      V.lg_x = lr + 2 * M;
+      V.lg_y = lr + 3 * M;
+      V.lrn = lr + 4 * M;
+      V.pick = pick + q * M;
+    }
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < ns; k += blockDim.x) {
+    const int cx = k % CW, cy = k / CW;
+    const int xr = tl.x0 + cx - 2, yr = tl.y0 + cy - 2;
+    const int xm = wrap_or_clamp(xr, nx, px), ym = wrap_or_clamp(yr, ny, py);
+    const int n = ym * nx + xm;
+    const bool solid = P.V[0].sol[n] != 0, beyond = (!px && xm != xr) || (!py && ym != yr);
+    s_node[k] = n;
+    s_mask[k] = P.V[0].nbm[n];
+    s_kind[k] = uint8_t((solid ? 1 : 0) | (beyond ? 2 : 0));
+    s_f[0][k] = s_f[1][k] = s_q[0][k] = s_q[1][k] = s_q[2][k] = s_acc[0][k] = s_acc[1][k] = R(0.0);
+    if (solid && cx >= 1 && cx < CW - 1 && cy >= 1 && cy < CH - 1) {
+      const int m = atomicAdd(&s_nlist, 1);
+      s_list[m] = uint16_t(k);
+      s_ref[m] = uint16_t(k + (py ? 0 : ym - yr) * CW + (px ? 0 : xm - xr));
+      R den = R(0.0);
+      for (int b = 1; b < 9; ++b)
+        if (!mask_bit(s_mask[k], b)) den = radd(den, wgt<R>(b));
+      s_den[m] = den;
+    }
+  }
+  __syncthreads();
+  const int nlist = s_nlist;
+  const bool solid = mine && (s_kind[c] & 1);
+  // an open column's nodes are also read through the ghost column beyond it
+  const int ghost = !mine || !inout ? 0 : (x == 0 ? -1 : (x == nx - 1 ? 1 : 0));
+
+  unsigned phase = P.base;
+  // the end of a stage: false once a wait of some thread of the block ran out
+  auto arrive = [&] {
+    __syncthreads();
+    ++phase;
+    if (threadIdx.x == 0) {
+      __threadfence();
+      flag_release(P.progress + blockIdx.x * kRunFlagStride, phase);
+    }
+  };
+  auto wait = [&]() -> bool {
+    bool lost = false;
+    for (int j = threadIdx.x; j < tl.nnb; j += blockDim.x) {
+      const unsigned* p = P.progress + P.nb[tl.nb0 + j] * kRunFlagStride;
+      int polls = 0;
+      while (int(flag_acquire(p) - phase) < 0)
+        if (++polls >= P.poll_limit || ((polls & 1023) == 0 && *static_cast<volatile int*>(P.err) != 0)) {
+          lost = true;
+          break;
+        }
+    }
+    if (__syncthreads_or(lost)) {
+      if (threadIdx.x == 0) atomicOr(P.err, ERR_TIMEOUT);
+      return false;
+    }
+    return true;
+  };
+  auto sync = [&]() -> bool {
+    arrive();
+    return wait();
+  };
+  // ---- forward half: a field (nf components) on tile + 2, its virtual values on the solid slots
+  // of tile + 1 (the sums of read_field in its order)
+  auto fill = [&](const R* v0, const R* v1) {
+    for (int k = u; k < ns; k += half)
+      if (!(s_kind[k] & 1)) {
+        s_f[0][k] = __ldcg(v0 + s_node[k]);
+        if (v1) s_f[1][k] = __ldcg(v1 + s_node[k]);
+      }
+    half_sync(2, half);
+    for (int m = u; m < nlist; m += half) {
+      const int k = s_list[m], r = s_ref[m];
+      const unsigned msk = s_mask[k];
+      R n0 = R(0.0), n1 = R(0.0);
+#pragma unroll
+      for (int b = 1; b < 9; ++b)
+        if (!mask_bit(msk, b)) {
+          n0 = radd(n0, rmul(wgt<R>(b), s_f[0][r + ey(b) * CW + ex(b)]));
+          if (v1) n1 = radd(n1, rmul(wgt<R>(b), s_f[1][r + ey(b) * CW + ex(b)]));
+        }
+      const R den = s_den[m];
+      s_f[0][k] = den > R(0.0) ? rdiv(n0, den) : R(0.0);
+      if (v1) s_f[1][k] = den > R(0.0) ? rdiv(n1, den) : R(0.0);
+    }
+    half_sync(2, half);
+  };
+  auto fwd_grad = [&](const AdjDevT<R>& A) {
+    fill(A.rn, nullptr);
+    if (mine)
+      fwd_grad_body(A, i, u, A.flags[L.node_off + (long long)y * L.pitch + x],
+                    [&](int a) { return s_f[0][c + ey(a) * CW + ex(a)]; });
+  };
+  auto fwd_dn = [&](const AdjDevT<R>& A) {
+    fill(A.nxv, A.nyv);
+    if (mine)
+      fwd_dn_body(A, u, solid, [&](int a) { return s_f[0][c + ey(a) * CW + ex(a)]; },
+                  [&](int a) { return s_f[1][c + ey(a) * CW + ex(a)]; });
+  };
+  // ---- reverse half: what the readers of slot k (fluid nodes of the lattice) pass to it, of
+  // sources (s0, s1) = adjoints of (d_x, d_y); g: only through a ghost beside column x = 0 (-1)
+  // or nx - 1 (1), whose readers lie on that column
+  auto readers = [&](const R* s0, const R* s1, int k, int g) {
+    R v = R(0.0);
+#pragma unroll
+    for (int a = 1; a < 9; ++a) {
+      if (g && ex(a) != g) continue;
+      const int r = k - ey(a) * CW - ex(a);
+      v += R(3.0) * wgt<R>(a) * (ex(a) * s0[r] + ey(a) * s1[r]);
+    }
+    return v;
+  };
+  // sources to shared memory (nq arrays), then the solid nodes' totals for nc components
+  auto collect = [&](const R* q0, const R* q1, const R* q2, int nc) {
+    for (int k = u; k < ns; k += half)
+      if (s_kind[k] == 0) {
+        s_q[0][k] = __ldcg(q0 + s_node[k]);
+        s_q[1][k] = __ldcg(q1 + s_node[k]);
+        if (q2) s_q[2][k] = __ldcg(q2 + s_node[k]);
+      }
+    half_sync(3, half);
+    for (int m = u; m < nlist; m += half) {
+      const int k = s_list[m];
+      if (s_kind[k] & 2) continue;
+      const int xs = s_node[k] % nx;
+      const int g = !inout ? 0 : (xs == 0 ? -1 : (xs == nx - 1 ? 1 : 0));
+      const R den = s_den[m], r = den > R(0.0) ? R(1.0) / den : R(0.0);
+      for (int q = 0; q < nc; ++q) {
+        R v = readers(s_q[q], s_q[q + 1], k, 0);
+        if (g) v += readers(s_q[q], s_q[q + 1], k + g, g);
+        s_acc[q][k] = v * r;
+      }
+    }
+    half_sync(3, half);
+  };
+  // the adjoint of what this node's neighbours read of it, component q
+  auto gather = [&](int q) {
+    R v = readers(s_q[q], s_q[q + 1], c, 0);
+    if (ghost) v += readers(s_q[q], s_q[q + 1], c + ghost, ghost);
+    const unsigned msk = s_mask[c];
+    if (msk) {
+#pragma unroll
+      for (int b = 1; b < 9; ++b) {
+        const int k = c - ey(b) * CW - ex(b);
+        if (s_kind[k] == 1) v += wgt<R>(b) * s_acc[q][k];
+        if (ghost && ex(b) == ghost) {
+          const int k2 = c + ghost - ey(b) * CW - ex(b);
+          if (s_kind[k2] == 1) v += wgt<R>(b) * s_acc[q][k2];
+        }
+      }
+    }
+    return v;
+  };
+
+  // the two sets of forward intermediates take turns: step j reverses with set q while the
+  // intermediates of state j - 1 go to the other.  Sources of the gathers: set 0's scatter
+  // targets hold those of n (three arrays), set 1's those of rho^N (two).
+  const char* src = P.states + (P.ns - 1) * P.stride;
+  if (!rev && mine) fwd_local_body<R, true>(s_V[0], src, i, u);
+  if (!sync()) return;
+  if (!rev) fwd_grad(s_V[0]);
+  if (!sync()) return;
+  if (!rev) fwd_dn(s_V[0]);
+  // the node's parameter adjoints, accumulated in double while the block waits
+  double p_sigma = 0.0, p_hR = 0.0, p_hB = 0.0, p_theta = 0.0;
+  const unsigned msk = mine ? s_mask[c] : 0u;
+  __syncthreads();
+  const R* lam_next = P.lam_next;
+  R* lam = P.lam;
+  int q = 0;
+#pragma unroll 1
+  for (int j = P.ns - 1; j >= 0; --j) {
+    const AdjDevT<R>& A = s_V[q];
+    const AdjDevT<R>& B = s_V[q ^ 1];
+    const bool fwd = !rev && j > 0;
+    src -= P.stride;
+    R ds = R(0.0), dR = R(0.0), dB = R(0.0), dt = R(0.0);
+    if (rev && mine)
+      adj_collide_body<R, true>(A, lam_next, i, u, solid, msk, ds, dR, dB, P.V[0].lnt_x, P.V[0].lnt_y, P.V[0].lrnt);
+    if (fwd && mine) fwd_local_body<R, true>(B, src, i, u);
+    arrive();
+    p_sigma += ds;
+    p_hR += dR;
+    p_hB += dB;
+    if (!wait()) return;
+    if (rev) {
+      collect(P.V[0].lnt_x, P.V[0].lnt_y, P.V[0].lrnt, 2);
+      if (mine) {
+        R lrx, lry;
+        adj_normal_body(A, i, u, solid, gather(0), gather(1), lrx, lry, dt);
+        P.V[1].lnt_x[i] = lrx;
+        P.V[1].lnt_y[i] = lry;
+      }
+    }
+    if (fwd) fwd_grad(B);
+    arrive();
+    p_theta += dt;
+    if (!wait()) return;
+    if (rev) {
+      collect(P.V[1].lnt_x, P.V[1].lnt_y, nullptr, 1);
+      if (mine) adj_rho_body(A, lam, i, u, solid, gather(0));
+    }
+    if (fwd) fwd_dn(B);
+    if (j > 0 && !sync()) return;
+    R* const l = lam;
+    lam = const_cast<R*>(lam_next);
+    lam_next = l;
+    q ^= 1;
+  }
+  if (rev && mine && !solid) {
+    P.V[0].p_sigma[i] += p_sigma;
+    P.V[0].p_hR[i] += p_hR;
+    P.V[0].p_hB[i] += p_hB;
+    P.V[0].p_theta[i] += p_theta;
+  }
 }
 
 // Seed for an objective J = sum_x c(x) rho^N(x) of the stored state: lam = dJ/d(state).
@@ -740,6 +1091,35 @@ cudaError_t adjoint_seed(const AdjDevT<R>& A, const R* c, bool red_mass, cudaStr
   return cudaGetLastError();
 }
 
+// 2 sets of 28 intermediates, 23 reverse values and 2 picks per node of the block
+template <typename R>
+static size_t reverse_smem(int threads) { return size_t(threads / 2) * ((2 * 28 + 23) * sizeof(R) + 2 * sizeof(int)); }
+
+template <typename R>
+cudaError_t launch_reverse(const RevRunT<R>& P, int ntiles, int threads, cudaStream_t st) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeCooperative;   // every block resident: they wait for one another
+  at[0].val.cooperative = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(unsigned(ntiles));
+  cfg.blockDim = dim3(unsigned(threads));
+  cfg.dynamicSmemBytes = reverse_smem<R>(threads);
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_reverse<R>, P);
+}
+template <typename R>
+cudaError_t reverse_blocks(int threads, int* per_sm) {
+  const cudaError_t e =
+      cudaFuncSetAttribute(k_reverse<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(reverse_smem<R>(threads)));
+  if (e != cudaSuccess) return e;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_reverse<R>, threads, reverse_smem<R>(threads));
+}
+template cudaError_t launch_reverse<double>(const RevRunT<double>&, int, int, cudaStream_t);
+template cudaError_t launch_reverse<float>(const RevRunT<float>&, int, int, cudaStream_t);
+template cudaError_t reverse_blocks<double>(int, int*);
+template cudaError_t reverse_blocks<float>(int, int*);
 template cudaError_t adjoint_forward<double>(const AdjDevT<double>&, cudaStream_t);
 template cudaError_t adjoint_forward<float>(const AdjDevT<float>&, cudaStream_t);
 template cudaError_t adjoint_step<double>(const AdjDevT<double>&, const AdjDevT<double>*, cudaStream_t);

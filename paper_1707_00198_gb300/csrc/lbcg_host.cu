@@ -106,6 +106,8 @@ struct lbcg_handle {
   bool run_planned = false;
   int run_tiles = 0;
   size_t run_smem = 0;
+  int run_threads = 0;
+  int run_nodes = 0, run_slots = 0;   // nodes of the largest tile, alone and with two all round
   char* d_run = nullptr;          // the plan's lists, one after another
   unsigned* d_progress = nullptr; // per tile: steps finished, counted from run_base
   unsigned run_base = 0;
@@ -443,8 +445,15 @@ lbcg_status plan_run(lbcg_handle* h) {
   if (fluid * (long long)(12 * cs + 8) > (long long)sms * blocks * (long long)budget) return LBCG_OK;
   RunPlan p;
   if (!build_run_plan(views, flags, h->ofb_host, blocks * sms, budget, cs, p)) return LBCG_OK;
+  for (const RunTile& t : p.tiles) {
+    h->run_nodes = std::max(h->run_nodes, t.tx * t.ty);
+    h->run_slots = std::max(h->run_slots, (t.tx + 4) * (t.ty + 4));
+  }
+  // blocks of 128 threads where the tiles are that small: they leave registers for a kernel on
+  // another stream (the adjoint's reverse sweep beside the recompute of a segment)
+  h->run_threads = cs == 4 && h->run_nodes <= 64 ? 128 : 256;
   int per_sm = 0;
-  CK(h, prepare_run(h->prec, p.smem, &per_sm));
+  CK(h, prepare_run(h->prec, h->run_threads, p.smem, &per_sm));
   if ((long long)per_sm * sms < (long long)p.tiles.size()) return LBCG_OK;
   size_t total = 0;
   std::vector<std::pair<const void*, size_t>> parts;
@@ -519,7 +528,7 @@ cudaError_t enqueue_run(lbcg_handle* h, int64_t* n) {
   a.pre = pre;
   a.nrep = int((*n - pre) / kGraphSteps);
   h->run_base += unsigned(*n);
-  cudaError_t e = launch_run(h->prec, a, h->run_tiles, h->run_smem, h->stream);
+  cudaError_t e = launch_run(h->prec, a, h->run_tiles, h->run_threads, h->run_smem, h->stream);
   if (e == cudaSuccess && h->prec >= 2 && a.nrep > 0) e = launch_sr_add(h->d_sr_epoch, uint32_t(a.nrep), h->stream);
   return e;
 }
@@ -1333,8 +1342,11 @@ lbcg_status adjoint_run(lbcg_handle* h, const lbcg_adjoint_spec* spec, lbcg_grad
     CK(h, cudaMemcpy(&ld, h->d_lats, sizeof(LatDev), cudaMemcpyDeviceToHost));
     ld.pop_off = 0;  // the adjoint reads states from its own buffers
     A.L = ld;
+    const LatConst<double> c = ld.consts<double>();
+    A.C = LatConst<R>{R(c.sigma),   R(c.beta),     R(c.s_e),       R(c.s_eps),     R(c.s_q),        R(c.rho0), R(c.u_in),
+                      R(c.rho_out), R(c.grad_eps), R(c.h_inv_nuR), R(c.h_inv_nuB), R(c.cos_theta)};
   }
-  A.N = N;
+  A.N = A.M = N;
   A.flags = h->d_flags;
   A.sol = sol;
   A.nbm = nbm;
@@ -1428,6 +1440,26 @@ lbcg_status adjoint_run(lbcg_handle* h, const lbcg_adjoint_spec* spec, lbcg_grad
   } graphs;
   R* const lam_a = lamA;
   R* const lam_b = lamB;
+  // the recompute as launches of the resident kernel, where the handle steps with it: its own
+  // progress words, since it may run beside the forward steps
+  // (progress2), and likewise the reverse sweep of a segment (progress3) where its blocks of
+  // rev_threads threads fit
+  unsigned *progress2 = nullptr, *progress3 = nullptr;
+  unsigned base2 = 0, base3 = 0;
+  int rev_threads = 0;
+  const bool resident = !h->sweep && h->run_tiles > 0 && h->poll_limit == kPollLimit && !h->profiling;
+  if (resident) {
+    const size_t pb = size_t(h->run_tiles) * kRunFlagStride * sizeof(unsigned);
+    if (!B.get(&progress2, pb) || !B.get(&progress3, pb)) return fail(LBCG_E_NOMEM, "adjoint buffers");
+    CK(h, cudaMemsetAsync(progress2, 0, pb, h->stream));
+    CK(h, cudaMemsetAsync(progress3, 0, pb, h->stream));
+    rev_threads = 2 * ((h->run_nodes + 31) / 32 * 32);
+    int dev = 0, sms = 0, per_sm = 0;
+    CK(h, cudaGetDevice(&dev));
+    CK(h, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    if (rev_threads <= kRevMaxThreads && h->run_slots <= kRevMaxSlots) CK(h, reverse_blocks<R>(rev_threads, &per_sm));
+    if ((long long)per_sm * sms < h->run_tiles) rev_threads = 0;
+  }
   auto enqueue_recompute = [&](int64_t ns, int b) -> cudaError_t {
     for (int64_t j = 1; j < ns; ++j) {
       LaunchStep p = make_launch(h, 0, nullptr, 0, h->ntiles);
@@ -1496,7 +1528,19 @@ lbcg_status adjoint_run(lbcg_handle* h, const lbcg_adjoint_spec* spec, lbcg_grad
     const int64_t ns = std::min<int64_t>(K, T - k * K);
     CK(h, cudaStreamWaitEvent(side.st, done[b], 0));
     CK(h, cudaMemcpyAsync(segs[b], reinterpret_cast<char*>(ckpt) + sb * k, sb, cudaMemcpyDeviceToDevice, side.st));
-    if (ns > 1) {
+    if (ns > 1 && resident) {
+      for (int64_t j = 0; j < ns - 1;) {
+        RunArgs a = h->run;
+        a.pool0 = reinterpret_cast<char*>(segs[b]) + sb * j;
+        a.stride = (long long)sb;
+        a.nsteps = int(std::min<int64_t>(ns - 1 - j, kRunMaxSteps));
+        a.progress = progress2;
+        a.base = base2;
+        base2 += unsigned(a.nsteps);
+        CK(h, launch_run(h->prec, a, h->run_tiles, h->run_threads, h->run_smem, side.st));
+        j += a.nsteps;
+      }
+    } else if (ns > 1) {
       const lbcg_status r = replay(0, ns, b, false, side.st);
       if (r != LBCG_OK) return r;
     }
@@ -1590,8 +1634,27 @@ lbcg_status adjoint_run(lbcg_handle* h, const lbcg_adjoint_spec* spec, lbcg_grad
       if (s != LBCG_OK) return s;
     }
     CK(h, cudaStreamWaitEvent(h->stream, ready[b], 0));
-    s = replay(1, ns, b, lam_in_a, h->stream);
-    if (s != LBCG_OK) return s;
+    if (rev_threads > 0) {
+      RevRunT<R> P{};
+      P.V[0] = V[0];
+      P.V[1] = V[1];
+      P.tiles = h->run.tiles;
+      P.nb = h->run.nb;
+      P.progress = progress3;
+      P.base = base3;
+      P.err = h->d_err;
+      P.poll_limit = kPollLimit;
+      P.states = reinterpret_cast<const char*>(segs[b]);
+      P.stride = (long long)sb;
+      P.ns = int(ns);
+      P.lam_next = lam_in_a ? lam_a : lam_b;
+      P.lam = lam_in_a ? lam_b : lam_a;
+      base3 += unsigned(3 * ns + 1);
+      CK(h, launch_reverse<R>(P, h->run_tiles, rev_threads, h->stream));
+    } else {
+      s = replay(1, ns, b, lam_in_a, h->stream);
+      if (s != LBCG_OK) return s;
+    }
     CK(h, cudaEventRecord(done[b], h->stream));
     if (ns & 1) lam_in_a = !lam_in_a;
   }
@@ -1602,6 +1665,8 @@ lbcg_status adjoint_run(lbcg_handle* h, const lbcg_adjoint_spec* spec, lbcg_grad
   CK(h, cudaMemcpyAsync(phB.data(), A.p_hB, N * 8, cudaMemcpyDeviceToHost, h->stream));
   CK(h, cudaMemcpyAsync(pth.data(), A.p_theta, N * 8, cudaMemcpyDeviceToHost, h->stream));
   CK(h, cudaStreamSynchronize(h->stream));
+  s = check_device_error(h);
+  if (s != LBCG_OK) return s;
   double gs = 0, ghR = 0, ghB = 0, gth = 0;
   for (int i = 0; i < N; ++i) {
     gs += ps[i];
@@ -1743,7 +1808,7 @@ lbcg_status lbcg_autotune(lbcg_handle* h, int32_t probe_steps, int32_t* schedule
         if (q) e = cudaEventRecord(e0, h->stream);
         a.base = h->run_base;
         h->run_base += unsigned(n);
-        if (e == cudaSuccess) e = launch_run(h->prec, a, h->run_tiles, h->run_smem, h->stream);
+        if (e == cudaSuccess) e = launch_run(h->prec, a, h->run_tiles, h->run_threads, h->run_smem, h->stream);
       }
       if (e == cudaSuccess) e = cudaEventRecord(e1, h->stream);
       for (int q = 0; q < 2 && e == cudaSuccess; ++q)

@@ -90,9 +90,9 @@ struct RunArgs {
     return sr_key(q < 0 ? epoch : epoch + uint32_t(nrep), step0 + uint32_t(s), pop_off);
   }
 };
-cudaError_t launch_run(int prec, const RunArgs& a, int ntiles, size_t smem, cudaStream_t st);
+cudaError_t launch_run(int prec, const RunArgs& a, int ntiles, int threads, size_t smem, cudaStream_t st);
 // sets the kernel's shared memory and asks how many of its blocks an SM holds
-cudaError_t prepare_run(int prec, size_t smem, int* per_sm);
+cudaError_t prepare_run(int prec, int threads, size_t smem, int* per_sm);
 cudaError_t launch_sr_add(uint32_t* epoch, uint32_t n, cudaStream_t st);
 
 cudaError_t launch_to_storage(int prec, const LatDev* lats, int lat, long long nn, const double* in,
@@ -122,7 +122,10 @@ cudaError_t launch_observables(const LatDev* lats, int lat, int nx, int ny, cons
 template <typename R>
 struct AdjDevT {
   LatDev L;
+  LatConst<R> C;
   int N;
+  int M;   // elements per plane of the arrays only a node's own threads use (fr, fb, rr, rb, gr*,
+           // gc*, dn, pick, lf_*, ln_*, lg_*, lrn): N, or a block's nodes in its shared memory
   const void* src;       // stored state (population pool of the lattice), FP64 or FP32
   int src_fp32;          // 1: the state is stored in FP32 (an FP32 forward)
   // |grad rho^N| at or below which the reverse sweep takes n = g/|g| as constant.  FP64
@@ -167,6 +170,32 @@ template <typename R>
 cudaError_t adjoint_forward(const AdjDevT<R>& A, cudaStream_t st);
 template <typename R>
 cudaError_t adjoint_step(const AdjDevT<R>& A, const AdjDevT<R>* B, cudaStream_t st);
+// A segment's reverse sweep as one cooperative launch (k_reverse): the states at `states`,
+// `stride` bytes apart, reversed from state ns - 1 to state 0; lam_next and lam take turns, so
+// that the result is in lam_next's array if ns is even, in lam's if it is odd.  Tiles and
+// neighbours of the resident step kernel's plan; progress words of its own, 3 ns + 1 phases from
+// base on.  `threads`: twice the nodes of the largest tile, rounded up to whole warps each.
+constexpr int kRevMaxThreads = 256;
+constexpr int kRevMaxSlots = 512;   // nodes of a tile plus two all round, at most
+template <typename R>
+struct RevRunT {
+  AdjDevT<R> V[2];
+  const RunTile* tiles;
+  const int* nb;
+  unsigned* progress;
+  unsigned base;
+  int* err;
+  int poll_limit;
+  const char* states;
+  long long stride;
+  int ns;
+  const R* lam_next;
+  R* lam;
+};
+template <typename R>
+cudaError_t launch_reverse(const RevRunT<R>& P, int ntiles, int threads, cudaStream_t st);
+template <typename R>
+cudaError_t reverse_blocks(int threads, int* per_sm);
 // seed lam = dJ/d(state): J = sum weight * rho^N (red_mass false) or the red mass (true)
 template <typename R>
 cudaError_t adjoint_seed(const AdjDevT<R>& A, const R* weight, bool red_mass, cudaStream_t st);

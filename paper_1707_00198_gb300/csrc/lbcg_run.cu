@@ -74,7 +74,7 @@ __device__ __forceinline__ T* carve(unsigned char*& p, size_t n) {
 template <typename S, int NT>
 __global__ void __launch_bounds__(NT, run_blocks(sizeof(typename Store<S>::T))) k_run(RunArgs A) {
   using T = typename Store<S>::T;
-  constexpr int kWallTeam = 128;   // threads that evaluate a tile's wall nodes beside its bulk nodes
+  constexpr int kWallTeam = NT / 2;   // threads that evaluate a tile's wall nodes beside its bulk nodes
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ LatDev sL;
   const RunTile tl = A.tiles[blockIdx.x];
@@ -392,50 +392,52 @@ __global__ void __launch_bounds__(NT, run_blocks(sizeof(typename Store<S>::T))) 
 
 __global__ void k_sr_add(uint32_t* epoch, uint32_t n) { *epoch += n; }
 
-constexpr int kRunThreads = 256;
-
 template <typename S>
-cudaError_t launch(const RunArgs& a, int ntiles, size_t smem, cudaStream_t st) {
+cudaError_t launch(const RunArgs& a, int ntiles, int threads, size_t smem, cudaStream_t st) {
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeCooperative;   // every block resident: they wait for one another
   at[0].val.cooperative = 1;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(unsigned(ntiles));
-  cfg.blockDim = dim3(kRunThreads);
+  cfg.blockDim = dim3(unsigned(threads));
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_run<S, kRunThreads>, a);
+  return threads == 128 ? cudaLaunchKernelEx(&cfg, k_run<S, 128>, a) : cudaLaunchKernelEx(&cfg, k_run<S, 256>, a);
 }
 
-template <typename S>
-cudaError_t prepare(size_t smem, int* per_sm) {
-  cudaError_t e = cudaFuncSetAttribute(k_run<S, kRunThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-  if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_run<S, kRunThreads>, kRunThreads, smem);
+template <typename K>
+cudaError_t prepare_k(K* k, int threads, size_t smem, int* per_sm) {
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k, threads, smem);
   return e;
+}
+template <typename S>
+cudaError_t prepare(int threads, size_t smem, int* per_sm) {
+  return threads == 128 ? prepare_k(k_run<S, 128>, threads, smem, per_sm)
+                        : prepare_k(k_run<S, 256>, threads, smem, per_sm);
 }
 
 }  // namespace
 
-cudaError_t launch_run(int prec, const RunArgs& a, int ntiles, size_t smem, cudaStream_t st) {
+cudaError_t launch_run(int prec, const RunArgs& a, int ntiles, int threads, size_t smem, cudaStream_t st) {
   cudaError_t e = cudaErrorInvalidValue;
   switch (prec) {
-    case 0: e = launch<double>(a, ntiles, smem, st); break;
-    case 1: e = launch<float>(a, ntiles, smem, st); break;
-    case 2: e = launch<__half>(a, ntiles, smem, st); break;
-    case 3: e = launch<__nv_bfloat16>(a, ntiles, smem, st); break;
+    case 0: e = launch<double>(a, ntiles, threads, smem, st); break;
+    case 1: e = launch<float>(a, ntiles, threads, smem, st); break;
+    case 2: e = launch<__half>(a, ntiles, threads, smem, st); break;
+    case 3: e = launch<__nv_bfloat16>(a, ntiles, threads, smem, st); break;
   }
   return e;
 }
 
-cudaError_t prepare_run(int prec, size_t smem, int* per_sm) {
+cudaError_t prepare_run(int prec, int threads, size_t smem, int* per_sm) {
   switch (prec) {
-    case 0: return prepare<double>(smem, per_sm);
-    case 1: return prepare<float>(smem, per_sm);
-    case 2: return prepare<__half>(smem, per_sm);
-    case 3: return prepare<__nv_bfloat16>(smem, per_sm);
+    case 0: return prepare<double>(threads, smem, per_sm);
+    case 1: return prepare<float>(threads, smem, per_sm);
+    case 2: return prepare<__half>(threads, smem, per_sm);
+    case 3: return prepare<__nv_bfloat16>(threads, smem, per_sm);
   }
   return cudaErrorInvalidValue;
 }
