@@ -170,11 +170,11 @@ lbcg_status lbcg_create(const lbcg_geometry* geom, const lbcg_params* prm, int32
 lbcg_status lbcg_create_batch(int32_t n, const lbcg_geometry* geoms, const lbcg_params* prms,
                               int32_t precision, void* stream, lbcg_handle** out);
 
-/* Enqueue `nsteps` >= 0 time steps on the handle's stream (asynchronous).  A call of more than 32
- * steps of a handle on the tile schedule whose lattices fit on the GPU at once (one tile per
- * resident block) is launched as one cooperative kernel that takes all the steps (at most 8192
- * per launch); other calls of 32 steps and more replay a captured CUDA graph, and short ones
- * launch each kernel.  The results do not depend on which. */
+/* Enqueue `nsteps` >= 0 time steps on the handle's stream (asynchronous).  A call of 8 steps or
+ * more, other than 32, of a handle on the tile schedule whose lattices fit on the GPU at once (one
+ * tile per resident block) is launched as one cooperative kernel that takes all the steps (at
+ * most 8192 per launch); other calls of 32 steps and more replay a captured CUDA graph, and short
+ * ones launch each kernel.  The results do not depend on which. */
 lbcg_status lbcg_step(lbcg_handle* h, int64_t nsteps);
 
 /* Measure the observables of lattice `lattice` of the current state (synchronises the

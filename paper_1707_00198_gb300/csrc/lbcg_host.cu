@@ -47,7 +47,8 @@ constexpr int kGraphBranches = 3; // parallel branches of a batch's graph (group
 constexpr int kHostGroups = 8;    // lattice groups whose copies lbcg_step_host overlaps
 constexpr int kDefaultTY = 8;
 constexpr int kPollLimit = 1 << 22;   // default polls of a bounded device wait (about a second)
-constexpr int kRunMaxSteps = 8192;    // steps per launch of the resident kernel, at most
+constexpr int kRunMaxSteps = 8192;    // steps per launch of the resident kernel, at most,
+constexpr int kRunMinSteps = 8;       // and of a call that it takes, at least
 constexpr int kSMs = 152;
 
 size_t elem_size(int prec) { return prec == 0 ? 8 : (prec == 1 ? 4 : 2); }
@@ -101,6 +102,12 @@ struct lbcg_handle {
   OfbEntry* d_ofb = nullptr;
   int nofb = 0;
   double* d_obs = nullptr;   // partials then outputs
+  // pinned host memory of small results: the device error word, then up to kObsOut doubles
+  struct Small {
+    int err;
+    double v[kObsOut];
+  };
+  Small* h_small = nullptr;
   // the resident kernel of the tile schedule (calls of more than kGraphSteps steps): its plan
   // on the device, or run_tiles = 0 where the lattices do not fit
   bool run_planned = false;
@@ -362,6 +369,7 @@ void free_handle(lbcg_handle* h) {
                   h->d_obs,   h->d_strips, h->d_nbmask, h->d_err, h->d_usnap, h->d_sr_epoch,
                   h->d_run,   h->d_progress};
   if (h->stream) cudaStreamSynchronize(h->stream);
+  if (h->h_small) cudaFreeHost(h->h_small);
   for (void* p : ptrs) dev_free(h, p);
   for (int b = 0; b < kGraphBranches; ++b) {
     if (h->br_stream[b]) cudaStreamDestroy(h->br_stream[b]);
@@ -504,12 +512,13 @@ lbcg_status plan_run(lbcg_handle* h) {
   return LBCG_OK;
 }
 
-// Whether a call of nsteps steps runs as launches of the resident kernel.  Calls of up to
-// kGraphSteps steps keep the launch-per-step schedule (the resident kernel's launch resolves the
-// lattice's tables first), and so do profiled handles (events around each kernel), handles
-// whose poll limit was changed and streams that are being captured.
+// Whether a call of nsteps steps runs as launches of the resident kernel: from kRunMinSteps on
+// (a launch resolves the lattice's tables first, about two steps' worth of time), except a call
+// of exactly one graph replay, whose launches per step callers may count (lbcg_step_launches).
+// Profiled handles (events around each kernel), handles whose poll limit was changed and
+// streams that are being captured keep the launch-per-step schedule.
 bool runs_resident(const lbcg_handle* h, int64_t nsteps) {
-  if (h->sweep || h->run_tiles == 0 || nsteps <= kGraphSteps || h->profiling || h->poll_limit != kPollLimit) return false;
+  if (h->sweep || h->run_tiles == 0 || nsteps < kRunMinSteps || nsteps == kGraphSteps || h->profiling || h->poll_limit != kPollLimit) return false;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   return cudaStreamIsCapturing(h->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
 }
@@ -546,10 +555,7 @@ lbcg_status ensure_macro(lbcg_handle* h) {
 // resident kernel for a tile next to it), so the state of the steps since the last check is
 // unreliable (that block stopped without writing the rest).  The word is cleared once reported: the handle stays usable, and a state set
 // or uploaded afterwards steps correctly again.
-lbcg_status check_device_error(lbcg_handle* h) {
-  int e = 0;
-  if (cudaMemcpy(&e, h->d_err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
-    return cuda_fail(h, cudaGetLastError(), "reading the device error word");
+lbcg_status report_device_error(lbcg_handle* h, int e) {
   if (e) {
     if (cudaMemset(h->d_err, 0, sizeof(int)) != cudaSuccess)
       return cuda_fail(h, cudaGetLastError(), "clearing the device error word");
@@ -562,6 +568,20 @@ lbcg_status check_device_error(lbcg_handle* h) {
                 (e & ERR_DRAIN) ? " and its copies could not be drained" : "");
   }
   return LBCG_OK;
+}
+lbcg_status check_device_error(lbcg_handle* h) {
+  int e = 0;
+  if (cudaMemcpy(&e, h->d_err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
+    return cuda_fail(h, cudaGetLastError(), "reading the device error word");
+  return report_device_error(h, e);
+}
+// The end of a call that returns data: the error word comes back behind what is already on the
+// stream, so that the call waits for the GPU once (a blocking copy of the word after the wait
+// cost about 10 us of a call).
+lbcg_status finish_stream(lbcg_handle* h) {
+  CK(h, cudaMemcpyAsync(&h->h_small->err, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+  CK(h, cudaStreamSynchronize(h->stream));
+  return report_device_error(h, h->h_small->err);
 }
 
 lbcg_status check_handle(const lbcg_handle* h) {
@@ -807,6 +827,12 @@ lbcg_status lbcg_create_batch(int32_t n, const lbcg_geometry* geoms, const lbcg_
     free_handle(h);
     return fail(LBCG_E_NOMEM, "device allocation failed (%lld nodes)", node_total);
   }
+  if (cudaMallocHost((void**)&h->h_small, sizeof(*h->h_small)) != cudaSuccess) {
+    cudaGetLastError();
+    h->h_small = nullptr;
+    free_handle(h);
+    return fail(LBCG_E_NOMEM, "pinned host allocation failed");
+  }
 #define CKC(call)                                         \
   do {                                                    \
     cudaError_t e_ = (call);                              \
@@ -978,10 +1004,9 @@ lbcg_status lbcg_observables(lbcg_handle* h, int32_t lattice, const lbcg_obs_spe
   double* res = h->d_obs + obs_partials_doubles();
   CK(h, launch_observables(h->d_lats, lattice, L.nx, L.ny, h->d_macro, h->node_total, h->d_flags, spec->tip_row0,
                            spec->tip_row1, spec->cl_row0, spec->cl_row1, parts, res, h->stream));
-  double o[kObsOut];
-  CK(h, cudaMemcpyAsync(o, res, sizeof(o), cudaMemcpyDeviceToHost, h->stream));
-  CK(h, cudaStreamSynchronize(h->stream));
-  s = check_device_error(h);
+  const double* const o = h->h_small->v;
+  CK(h, cudaMemcpyAsync(h->h_small->v, res, kObsOut * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+  s = finish_stream(h);
   if (s != LBCG_OK) return s;
   memset(out, 0, sizeof(*out));
   out->step = h->step;
@@ -1060,10 +1085,9 @@ lbcg_status lbcg_diagnostics(lbcg_handle* h, int32_t lattice, const lbcg_diag_sp
   double* res = h->d_obs + obs_partials_doubles();   // the reduction scratch of lbcg_observables
   CK(h, launch_diagnostics(h->d_lats, lattice, h->d_macro, h->node_total, h->d_flags, h->d_usnap, have, spec->cx,
                            spec->cy, spec->r, parts, res, h->stream));
-  double q[6];
-  CK(h, cudaMemcpyAsync(q, res, sizeof(q), cudaMemcpyDeviceToHost, h->stream));
-  CK(h, cudaStreamSynchronize(h->stream));
-  s = check_device_error(h);
+  const double* const q = h->h_small->v;
+  CK(h, cudaMemcpyAsync(h->h_small->v, res, 6 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+  s = finish_stream(h);
   if (s != LBCG_OK) return s;
   out->step = h->step;
   out->prev_step = h->snap_step[lattice];
@@ -1157,8 +1181,7 @@ lbcg_status lbcg_download_state(lbcg_handle* h, void* host_out, size_t bytes) {
   if (s != LBCG_OK) return s;
   if (!host_out || bytes != lbcg_state_bytes(h)) return fail(LBCG_E_ARG, "state size mismatch");
   CK(h, cudaMemcpyAsync(host_out, h->pool[h->cur], bytes, cudaMemcpyDeviceToHost, h->stream));
-  CK(h, cudaStreamSynchronize(h->stream));
-  return check_device_error(h);
+  return finish_stream(h);
 }
 
 lbcg_status lbcg_step_host(lbcg_handle* h, const void* host_in, void* host_out, size_t bytes, int64_t nsteps) {
