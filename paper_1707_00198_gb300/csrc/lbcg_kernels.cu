@@ -773,10 +773,14 @@ __global__ void __launch_bounds__(NTH, sizeof(typename Store<S>::T) == 4 ? 1024 
 //  - one thread issues bulk copies (cp.async.bulk, completing on an mbarrier) of row r + 1's
 //    32-node population segments and of its flag and neighbour-mask bytes into the other of
 //    two shared-memory slots while row r is processed; every thread waits with a bound;
-//  - stage 1 keeps what the collision of the row needs, the nine totals f_a = f_a,R + f_a,B
-//    and (rho_R, rho_B), in registers until the end of the iteration and then in a two-row
+//  - stage 1 keeps what the collision of the row needs, the nine totals f_a = f_a,R + f_a,B,
+//    (rho_R, rho_B) and rho^N, in registers until the end of the iteration and then in a two-row
 //    ring in shared memory that only the owning thread reads, so the collision two rows later
-//    neither reloads nor re-sums the populations; the thread's colour gradient is carried to
+//    neither reloads nor re-sums the populations; the ring's slots are three 16-byte words per
+//    thread, and the column's flags and masks stay in registers (the loop is bound by instruction
+//    issue: 64-channel step 0.2984 -> 0.2900 ms FP32, 0.2867 -> 0.2722 FP16 with both, and with
+//    the row offsets carried from row to row 0.2860 and 0.2655; the loop unrolled three times,
+//    for constant ring slots, is 20-40 % slower: the instruction caches); the thread's colour gradient is carried to
 //    that collision in registers (42 KB of shared memory per block: 5 blocks per SM in FP32);
 //  - the moment sums and the back-transform share partial sums (fewer FP32 operations);
 //  - 16-bit storage takes the totals straight from the stored deviations and forms the stored
@@ -836,7 +840,7 @@ __device__ __forceinline__ void staged_pair(const S* row, int a, float& lo, floa
 template <typename S, int NTH, bool kSchemeB>
 __global__ void __launch_bounds__(NTH, sizeof(S) == 4 ? kSweepFMinBlocks : kSweepFMinBlocks16) k_sweepf(SweepArgs A) {
   using T = float;
-  // rho^N / flag / neighbour-mask ring of rows r-2 .. r: row r takes row r-3's slot in stage 1
+  // rho^N / flag ring of rows r-2 .. r: row r takes row r-3's slot in stage 1
   // of iteration r; row r-3's last readers were stage 2 of iteration r-1 (other threads, before
   // that iteration's barriers) and stage 3 of iteration r-1 (only the owning thread)
   constexpr int RR = 3;
@@ -847,17 +851,15 @@ __global__ void __launch_bounds__(NTH, sizeof(S) == 4 ? kSweepFMinBlocks : kSwee
   __shared__ T srn[RR][NTH];
   __shared__ uint8_t sfl[RR][NTH];
   __shared__ V sn[RN][NTH];
-  __shared__ T sf[RF][9][NTH];
-  __shared__ V srb[RF][NTH];
+  // per thread: f_0 .. f_8, rho_R, rho_B and rho^N as three 16-byte words
+  __shared__ float4 sf[RF][3][NTH];
   __shared__ LatDev sL;
   // two staged rows of populations (dynamic shared memory): [slot][kStageSegs * kSeg]
   extern __shared__ __align__(128) unsigned char sraw_bytes[];
   S* sraw = reinterpret_cast<S*>(sraw_bytes);
   __shared__ __align__(8) uint64_t sbar[2];
-  // the staged rows' flags and neighbour-solid masks ([slot][0: flags, 1: mask][byte]), and the
-  // mask of rows r-2 .. r for the collision two rows later
+  // the staged rows' flags and neighbour-solid masks ([slot][0: flags, 1: mask][byte])
   __shared__ __align__(16) uint8_t sfg[2][2][NTH + 32];
-  __shared__ uint8_t snb[RR][NTH];
 
   const int4 sp = A.strips[blockIdx.x];
   const int t = threadIdx.x;
@@ -917,7 +919,8 @@ __global__ void __launch_bounds__(NTH, sizeof(S) == 4 ? kSweepFMinBlocks : kSwee
     return v < 0 ? 0 : (v >= ny ? ny - 1 : v);
   };
 
-  int ym3 = 0, ym2 = 0, ym1 = 0, ym0 = 0;
+  int ym2 = 0, ym1 = 0, ym0 = 0, yn = 0;   // lattice rows of sweep rows r - 2 .. r + 1
+  int rk3 = 0, rk2 = 0, rk1 = 0, rk0 = 0;   // and the population offsets of rows r - 3 .. r
   int s2 = 0, s1 = 1, s0 = 2;   // ring slots of rows r-2, r-1, r
   int n2 = 0, n1 = 1, n0 = 2;
   int q2 = 0, q1 = 1;   // f-total slots of rows r-2 and r-1
@@ -925,10 +928,14 @@ __global__ void __launch_bounds__(NTH, sizeof(S) == 4 ? kSweepFMinBlocks : kSwee
   // of row r until they take the slot of row r-2 at the end of the iteration, and the colour
   // gradient (stage 2, row r-1) until the collision of that row one iteration later
   T ft[9];
+  T rnt = T(0);
   V rbt = P::mk(T(0), T(0)), g_new = P::mk(T(0), T(0)), g_old = P::mk(T(0), T(0));
   bool ft_ok = false;
+  unsigned fm0 = F_SOLID, fm1 = F_SOLID, fm2 = F_SOLID;   // this column's flags | mask << 8 of rows r, r - 1, r - 2
   unsigned phase = 0;     // bit s: parity of the next completion of slot s
   bool lost = false;      // this thread's wait for a staged row ran out
+  __shared__ int s_lost;  // and some thread's of the block
+  if (t == 0) s_lost = 0;
   // issue the bulk copies of (mapped) row y into staging slot `slot` (one thread)
   auto stage_row = [&](int y, int slot) {
     S* d = sraw + slot * (kStageSegs * kSeg);
@@ -952,7 +959,14 @@ __global__ void __launch_bounds__(NTH, sizeof(S) == 4 ? kSweepFMinBlocks : kSwee
     mbar_init_fence();
   }
   __syncthreads();
-  if (t == 0) stage_row(map_row(yrow(ys - 2)), (ys - 2) & 1);
+  // the rows before the first: their products are read by the first pushes' addresses only
+  ym1 = map_row(yrow(ys - 4));
+  ym0 = map_row(yrow(ys - 3));
+  rk2 = map_row(yrow(ys - 5)) * rowseg;
+  rk1 = ym1 * rowseg;
+  rk0 = ym0 * rowseg;
+  yn = map_row(yrow(ys - 2));
+  if (t == 0) stage_row(yn, (ys - 2) & 1);
 
   // one row of the sweep; false once some thread of the block lost its wait for the row
   auto body = [&](const int r) -> bool {
@@ -965,36 +979,38 @@ __global__ void __launch_bounds__(NTH, sizeof(S) == 4 ? kSweepFMinBlocks : kSwee
       q2 = q1;
       q1 = tq;
       g_old = g_new;
-      if (r == ys - 2) {
-        ym3 = map_row(yrow(r - 3));
-        ym2 = map_row(yrow(r - 2));
-        ym1 = map_row(yrow(r - 1));
-      } else {
-        ym3 = ym2;
-        ym2 = ym1;
-        ym1 = ym0;
-      }
-      ym0 = map_row(yrow(r));
+      fm2 = fm1;
+      fm1 = fm0;
+      ym2 = ym1;
+      ym1 = ym0;
+      ym0 = yn;
+      rk3 = rk2;
+      rk2 = rk1;
+      rk1 = rk0;
+      rk0 = ym0 * rowseg;
     }
     // the next row's populations (bulk copy) and flag travel while this row is processed;
     // its slot held row r - 1, whose last reader finished before the previous barriers
     if (r + 1 <= ye + 1) {
-      const int y = map_row(yrow(r + 1));
-      if (t == 0) stage_row(y, (r + 1) & 1);
+      yn = map_row(yrow(r + 1));
+      if (t == 0) stage_row(yn, (r + 1) & 1);
     }
     const int p = r - 2;
-    const bool collide = p >= ys && interior && !(sfl[s2][t] & F_SOLID);
-    const uint8_t mask = collide ? snb[s2][t] : 0;
+    const bool collide = p >= ys && interior && !(fm2 & F_SOLID);
+    const unsigned mask = fm2 >> 8;
     // ---- stage 1: rho^N, totals and colour densities of row r
     {
       T v = T(0);
       const int slot = r & 1;
       // (after a lost wait this row's values are garbage: the block stops at the barrier below)
-      if (!mbar_wait(&sbar[slot], (phase >> slot) & 1u, A.poll_limit)) lost = true;
+      if (!mbar_wait(&sbar[slot], (phase >> slot) & 1u, A.poll_limit)) {
+        lost = true;
+        s_lost = 1;
+      }
       phase ^= 1u << slot;
       const bool fl_ok = fo >= 0 || checked(in_extent((long long)ym0 * pitch + xm, 1, node_n), err);
       const uint8_t f_r = fo >= 0 ? sfg[slot][0][fo] : (fl_ok ? fl[ym0 * pitch + xm] : uint8_t(F_SOLID));
-      snb[s0][t] = fo >= 0 ? sfg[slot][1][fo] : (fl_ok ? nbm[ym0 * pitch + xm] : uint8_t(0));
+      fm0 = f_r | unsigned(fo >= 0 ? sfg[slot][1][fo] : (fl_ok ? nbm[ym0 * pitch + xm] : uint8_t(0))) << 8;
       if (!(f_r & F_SOLID)) {
         T sr, sb;
         bool done = false;
@@ -1030,7 +1046,7 @@ __global__ void __launch_bounds__(NTH, sizeof(S) == 4 ? kSweepFMinBlocks : kSwee
             decode<S, T>(lo, hi, wgt<T>(a) * r0, fr[a], fb[a]);
           }
         } else if (checked(in_extent((long long)ym0 * rowseg + colk[1], 8 * kDir + 2, pop_n), err)) {
-          load_raw<S>(src + ym0 * rowseg + colk[1], r0, fr, fb);
+          load_raw<S>(src + rk0 + colk[1], r0, fr, fb);
         } else {
 #pragma unroll
           for (int a = 0; a < 9; ++a) fr[a] = fb[a] = T(0);
@@ -1049,12 +1065,14 @@ __global__ void __launch_bounds__(NTH, sizeof(S) == 4 ? kSweepFMinBlocks : kSwee
         v = sb == T(0) ? T(1) : (sr == T(0) ? T(-1) : w);
       }
       ft_ok = !(f_r & F_SOLID);
+      rnt = v;
       srn[s0][t] = v;
       sfl[s0][t] = f_r;
     }
     // every thread has seen row r, or the block stops here (before it writes anything of
-    // this row or the rows after it)
-    if (__syncthreads_or(lost)) return false;
+    // this row or the rows after it; a thread ahead sets s_lost again only after the next barrier)
+    __syncthreads();
+    if (s_lost) return false;
     // ---- stage 2: grad rho^N and n of row r - 1
     {
       const int tn = n2;
@@ -1117,12 +1135,10 @@ __global__ void __launch_bounds__(NTH, sizeof(S) == 4 ? kSweepFMinBlocks : kSwee
     __syncthreads();
     // ---- stage 3: collide and push row p = r - 2; then row r's totals take row p's slot
     if (collide) {
-    const uint8_t myf = sfl[s2][t];
-    T f[9];
-#pragma unroll
-    for (int a = 0; a < 9; ++a) f[a] = sf[q2][a][t];
-    const V rb = srb[q2][t];
-    const T rhoR = rb.x, rhoB = rb.y, rn = srn[s2][t];
+    const unsigned myf = fm2;
+    const float4 w0 = sf[q2][0][t], w1 = sf[q2][1][t], w2 = sf[q2][2][t];
+    const T f[9] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w, w2.x};
+    const T rhoR = w2.y, rhoB = w2.z, rn = w2.w;
     // grad n (Eq. 28), curvature (Eq. 13), force (Eq. 10)
     const V* nm = sn[down ? n0 : n2];   // n of rows y - 1, y, y + 1
     const V* n0v = sn[n1];
@@ -1214,8 +1230,8 @@ __global__ void __launch_bounds__(NTH, sizeof(S) == 4 ? kSweepFMinBlocks : kSwee
     pert[8] = c2 * (nxo - nyo);
     pert[7] = -pert[5];
     pert[6] = -pert[8];
-    const int kn = ym2 * rowseg + colk[1];
-    const int rowk[3] = {(down ? ym1 : ym3) * rowseg, ym2 * rowseg, (down ? ym3 : ym1) * rowseg};   // y - 1, y, y + 1
+    const int kn = rk2 + colk[1];
+    const int rowk[3] = {down ? rk1 : rk3, rk2, down ? rk3 : rk1};   // y - 1, y, y + 1
     uint32_t srh = 0;
     if constexpr (Store<S>::kDeviation) srh = sr_node(srk, kn);
     const T cg = fmaf(cR, T(2.0f * kK), T(-kK));   // K (2 cR - 1), deviation storage only
@@ -1230,29 +1246,42 @@ __global__ void __launch_bounds__(NTH, sizeof(S) == 4 ? kSweepFMinBlocks : kSwee
         store_pair<S>(q, oR, fp[a] - oR, wgt<T>(a) * r0);
       }
     };
-    if (mask == 0 && !(myf & F_EDGE)) {
+    // A bulk node's targets are its nine neighbours; next to a solid node the opposite slot of the
+    // node itself (half-way bounce-back), beyond an open edge nothing.  FP32: one run of stores whose
+    // targets a wall node corrects first, 0.2860 -> 0.2797 ms per 64-channel step; 16-bit storage
+    // keeps two runs (one costs it registers: 0.2655 -> 0.311 ms).
+    const bool okx[3] = {px || cx - 1 >= 0, true, px || cx + 1 < nx};   // (closed rows are solid)
+    const bool bulk = mask == 0 && !(myf & F_EDGE);
+    auto target = [&](int a) { return rowk[ey(a) + 1] + colk[ex(a) + 1] + a * kDir; };
+    if constexpr (!Store<S>::kDeviation) {
+      int k[9];
 #pragma unroll
-      for (int a = 0; a < 9; ++a) emit(dst + rowk[ey(a) + 1] + colk[ex(a) + 1] + a * kDir, a);
+      for (int a = 0; a < 9; ++a) k[a] = target(a);
+      if (!bulk) {
+#pragma unroll
+        for (int a = 1; a < 9; ++a) {
+          if (mask & (1u << (a - 1))) k[a] = kn + opp(a) * kDir;
+          if (!okx[ex(a) + 1]) k[a] = -1;
+        }
+      }
+#pragma unroll
+      for (int a = 0; a < 9; ++a)
+        if (a == 0 || k[a] >= 0) emit(dst + k[a], a);
+    } else if (bulk) {
+#pragma unroll
+      for (int a = 0; a < 9; ++a) emit(dst + target(a), a);
     } else {
-      const bool okx[3] = {px || cx - 1 >= 0, true, px || cx + 1 < nx};
-      const int yp = yrow(p);
-      const bool oky[3] = {py || yp - 1 >= 0, true, py || yp + 1 < ny};
 #pragma unroll
       for (int a = 0; a < 9; ++a) {
-        int k = kn + a * kDir;
-        if (a != 0) {
-          if (!(okx[ex(a) + 1] && oky[ey(a) + 1])) continue;
-          if (mask & (1u << (a - 1))) k = kn + opp(a) * kDir;
-          else k = rowk[ey(a) + 1] + colk[ex(a) + 1] + a * kDir;
-        }
-        emit(dst + k, a);
+        if (!okx[ex(a) + 1]) continue;
+        emit(dst + (a != 0 && (mask & (1u << (a - 1))) ? kn + opp(a) * kDir : target(a)), a);
       }
     }
     }
     if (ft_ok) {
-#pragma unroll
-      for (int a = 0; a < 9; ++a) sf[q2][a][t] = ft[a];
-      srb[q2][t] = rbt;
+      sf[q2][0][t] = make_float4(ft[0], ft[1], ft[2], ft[3]);
+      sf[q2][1][t] = make_float4(ft[4], ft[5], ft[6], ft[7]);
+      sf[q2][2][t] = make_float4(ft[8], rbt.x, rbt.y, rnt);
     }
     return true;
   };
