@@ -168,7 +168,12 @@ __global__ void __launch_bounds__(kWallThreads, sizeof(S) == 8 ? 3 : 5) k_wall(c
           zou_he<T>(x, sL.nx, inlet_u<T>(sL, y), T(sL.rho_out), fr[v], fb[v]);
         }
         T rR, rB;
-        val[i] = colour_indicator(fr[v], fb[v], rR, rB);
+        if constexpr (sizeof(T) == 8) {
+          T irho;
+          val[i] = indicator(fr[v], fb[v], rR, rB, irho);
+        } else {
+          val[i] = colour_indicator(fr[v], fb[v], rR, rB);
+        }
       }
     }
   }
@@ -186,7 +191,7 @@ __global__ void __launch_bounds__(kWallThreads, sizeof(S) == 8 ? 3 : 5) k_wall(c
           num = radd(num, rmul(wgt<T>(b), val[q.i[b - 1]]));
           den = radd(den, wgt<T>(b));
         }
-      v = rdiv(num, den);
+      v = mean_of(num, mean_factor(den));
     }
     val[G.nband + j] = v;
   }
@@ -332,8 +337,8 @@ __global__ void __launch_bounds__(32 * TY, sizeof(typename Store<S>::T) == 4 ? 1
         }
       }
       if (den > T(0)) {
-        nxv = rdiv(vx, den);
-        nyv = rdiv(vy, den);
+        nxv = mean_of(vx, mean_factor(den));
+        nyv = mean_of(vy, mean_factor(den));
       }
     }
     snx[cy * W1 + cx] = nxv;
@@ -386,6 +391,7 @@ __global__ void __launch_bounds__(32 * TY, sizeof(typename Store<S>::T) == 4 ? 1
     A.macro[3 * NTOT + k] = double(uy);
     return;
   } else {
+    if constexpr (sizeof(T) == 8) relax_rest(m, rho, K);
     T fp[9];
     collide_node<T>(f, m, rho, irho, viscous_rate<T>(rn, K), Fx, Fy, K, fp);
     const Recolour<T> rc(rhoR, rhoB, irho, nxo, nyo, K);

@@ -209,6 +209,13 @@ struct Moments {
   }
 };
 
+// FP64: the e and eps moments relaxed towards their values at rest and weighted, what the
+// collision needs of them apart from u and F
+__device__ __forceinline__ void relax_rest(Moments<double>& m, double rho, const Collide<double>& c) {
+  m.e = fma_(c.e1, m.e, rmul(c.e3, rho));
+  m.eps = fma_(c.p1, m.eps, rmul(c.p3, rho));
+}
+
 // s_v = 1/tau_v = 1/(3 nu + 1/2) (Eq. 5) with the harmonic viscosity of Eq. 18
 template <typename T>
 __device__ __forceinline__ T viscous_rate(T rn, const Collide<T>& c) {
@@ -226,7 +233,7 @@ __device__ __forceinline__ void velocity(const Moments<T>& m, T irho, T Fx, T Fy
 }
 
 // MRT collision with Guo forcing (Eq. 1-9): f' from the totals f (FP32; unused in FP64) or their
-// moments.  M^-1 = M^T diag(1/9, 1/36, 1/36, 1/6, 1/12, 1/6, 1/12, 1/4, 1/4); s_rho = s_j = 1
+// moments (FP64: after relax_rest).  M^-1 = M^T diag(1/9, 1/36, 1/36, 1/6, 1/12, 1/6, 1/12, 1/4, 1/4); s_rho = s_j = 1
 // (Eq. 6), so the momentum changes by exactly F.
 template <typename T>
 __device__ __forceinline__ void collide_node(const T* f, const Moments<T>& m, T rho, T irho, T sv, T Fx, T Fy,
@@ -237,8 +244,8 @@ __device__ __forceinline__ void collide_node(const T* f, const Moments<T>& m, T 
     const T yy = rmul(Jy, uy), uyF = rmul(uy, Fy);
     const T uu = fma_(Jx, ux, yy), dd = fma_(Jx, ux, -yy);             // rho u.u, rho (ux^2 - uy^2)
     const T uF = fma_(ux, Fx, uyF), dF = fma_(ux, Fx, -uyF), cF = fma_(ux, Fy, rmul(uy, Fx));
-    const T ae = fma_(c.e1, m.e, fma_(c.e2, uu, fma_(c.e3, rho, rmul(c.e4, uF))));
-    const T ap = fma_(c.p1, m.eps, fma_(c.p2, uu, fma_(c.p3, rho, rmul(c.p4, uF))));
+    const T ae = fma_(c.e2, uu, fma_(c.e4, uF, m.e));
+    const T ap = fma_(c.p2, uu, fma_(c.p4, uF, m.eps));
     const T aqx = fma_(c.q1, m.qx, fma_(c.q2, Jx, rmul(c.q3, Fx)));
     const T aqy = fma_(c.q1, m.qy, fma_(c.q2, Jy, rmul(c.q3, Fy)));
     const T ajx = rmul(radd(m.jx, Fx), T(1.0 / 6.0)), ajy = rmul(radd(m.jy, Fy), T(1.0 / 6.0));
@@ -318,7 +325,7 @@ struct Recolour {
 };
 
 // Virtual value of Eq. 29 on an outermost solid node: the weighted mean of `val` over its fluid
-// neighbours (local indices q, kWallNone where the neighbour is solid); den: virtual_weight(q)
+// neighbours (local indices q, kWallNone where the neighbour is solid); factor: mean_factor(virtual_weight(q))
 template <typename T>
 __device__ __forceinline__ T virtual_weight(const uint16_t q[8]) {
   T den = T(0);
@@ -327,13 +334,25 @@ __device__ __forceinline__ T virtual_weight(const uint16_t q[8]) {
     if (q[b - 1] != kWallNone) den = radd(den, wgt<T>(b));
   return den;
 }
+// What a sum over the fluid neighbours is divided by (FP32) or multiplied with (FP64: the
+// reciprocal, 1 operation instead of 9), from the weight
 template <typename T>
-__device__ __forceinline__ T virtual_value(const WallSten& q, const T* val, T den) {
+__device__ __forceinline__ T mean_factor(T den) {
+  if constexpr (sizeof(T) == 8) return rcp_(den);
+  else return den;
+}
+template <typename T>
+__device__ __forceinline__ T mean_of(T num, T factor) {
+  if constexpr (sizeof(T) == 8) return rmul(num, factor);
+  else return rdiv(num, factor);
+}
+template <typename T>
+__device__ __forceinline__ T virtual_value(const WallSten& q, const T* val, T factor) {
   T num = T(0);
 #pragma unroll
   for (int b = 1; b < 9; ++b)
     if (q.i[b - 1] != kWallNone) num = radd(num, rmul(wgt<T>(b), val[q.i[b - 1]]));
-  return rdiv(num, den);
+  return mean_of(num, factor);
 }
 
 // The two candidates of Eq. 34 on an outermost fluid node (rotations by +theta and -theta)
@@ -361,33 +380,54 @@ __device__ __forceinline__ void wall_normal_pair(T eps, int wetting, T f1, T f2,
   g = radd(g, r ? v6 : -v6);
   g = radd(g, -v(7));
   g = radd(g, r ? -v8 : v8);
-  g = rdiv(g, T(1.0 / 3.0));
+  if constexpr (sizeof(T) == 8) g = rmul(g, T(3));
+  else g = rdiv(g, T(1.0 / 3.0));
   auto other = [](T x) { return __shfl_xor_sync(0xFFFFFFFFu, x, 1); };
   T sq = rmul(g, g);
-  const T mag = rsqrt_(radd(sq, other(sq)));
-  const bool on = mag > eps;
-  const T es = rdiv(g, on ? mag : T(1)), eo = other(es);
   cg = g;
   n = T(0);
-  if (wetting == 2) {   // uniform over the block
-    if (on) n = es;     // no geometric correction: n from the raw gradient
-    return;
-  }
-  const T a1 = rsub(cx, r ? eo : es), b1 = rsub(cy, r ? es : eo);
-  const T d = rsqrt_(radd(rmul(a1, a1), rmul(b1, b1))), od = other(d);
-  const bool one = r ? od <= d : d <= od;
-  const T cc = rmul(mag, one ? f1 : f2);
-  sq = rmul(cc, cc);
-  const T m2 = rsqrt_(radd(sq, other(sq)));
-  if (on) {
-    cg = cc;
-    if (m2 > eps) n = rdiv(cc, m2);
+  if constexpr (sizeof(T) == 8) {   // as wall_normal's FP64 form
+    const T m2 = radd(sq, other(sq)), inv = rsqrt(m2), mag = rmul(m2, inv);
+    const bool on = mag > eps;
+    const T es = rmul(g, inv), eo = other(es);
+    if (wetting == 2) {
+      if (on) n = es;
+      return;
+    }
+    const T a1 = rsub(cx, r ? eo : es), b1 = rsub(cy, r ? es : eo);
+    const T d = radd(rmul(a1, a1), rmul(b1, b1)), od = other(d);
+    const T nf = (r ? od <= d : d <= od) ? f1 : f2;
+    if (on) {
+      cg = rmul(mag, nf);
+      n = nf;
+    }
+  } else {
+    const T mag = rsqrt_(radd(sq, other(sq)));
+    const bool on = mag > eps;
+    const T es = rdiv(g, on ? mag : T(1)), eo = other(es);
+    if (wetting == 2) {   // uniform over the block
+      if (on) n = es;     // no geometric correction: n from the raw gradient
+      return;
+    }
+    const T a1 = rsub(cx, r ? eo : es), b1 = rsub(cy, r ? es : eo);
+    const T d = rsqrt_(radd(rmul(a1, a1), rmul(b1, b1))), od = other(d);
+    const bool one = r ? od <= d : d <= od;
+    const T cc = rmul(mag, one ? f1 : f2);
+    sq = rmul(cc, cc);
+    const T m2 = rsqrt_(radd(sq, other(sq)));
+    if (on) {
+      cg = cc;
+      if (m2 > eps) n = rdiv(cc, m2);
+    }
   }
 }
 
 // Eq. 28 on an outermost fluid node from the shared values of its 8 neighbours, then the
-// contact-angle correction of Eq. 30-36 -> corrected gradient and unit normal.  The arithmetic
-// is rounding-exact in the oracle's order (directions 1..8, products w*phi then sign).
+// contact-angle correction of Eq. 30-36 -> corrected gradient and unit normal.  The sums run
+// in the oracle's order (directions 1..8, products w*phi then sign), so that a gradient exactly
+// along the wall's normal makes Eq. 35-36 an exact tie.  FP64 takes one reciprocal square root in
+// place of three square roots and seven divisions: it compares the squared distances (equal
+// whenever the distances of an exact tie are) and takes n = n_f (28 operations against 78).
 template <typename T>
 __device__ __forceinline__ void wall_normal(T eps, int wetting, T nsx, T nsy, T c, T s, const WallSten& q, const T* val,
                                             T& cgx, T& cgy, T& nx, T& ny) {
@@ -399,6 +439,30 @@ __device__ __forceinline__ void wall_normal(T eps, int wetting, T nsx, T nsy, T 
     if (ex(a) == -1) gx = radd(gx, -tt);
     if (ey(a) == 1) gy = radd(gy, tt);
     if (ey(a) == -1) gy = radd(gy, -tt);
+  }
+  if constexpr (sizeof(T) == 8) {
+    gx = rmul(gx, T(3));
+    gy = rmul(gy, T(3));
+    const T m2 = radd(rmul(gx, gx), rmul(gy, gy)), inv = rsqrt(m2), mag = rmul(m2, inv);
+    cgx = gx;
+    cgy = gy;
+    nx = ny = T(0);
+    if (!(mag > eps)) return;   // (also where m2 = 0)
+    const T esx = rmul(gx, inv), esy = rmul(gy, inv);
+    if (wetting == 2) {
+      nx = esx;
+      ny = esy;
+      return;
+    }
+    T f1x, f1y, f2x, f2y;
+    wall_candidates<T>(nsx, nsy, c, s, f1x, f1y, f2x, f2y);
+    const T a1 = rsub(f1x, esx), b1 = rsub(f1y, esy), a2 = rsub(f2x, esx), b2 = rsub(f2y, esy);
+    const bool one = radd(rmul(a1, a1), rmul(b1, b1)) <= radd(rmul(a2, a2), rmul(b2, b2));
+    nx = one ? f1x : f2x;
+    ny = one ? f1y : f2y;
+    cgx = rmul(mag, nx);
+    cgy = rmul(mag, ny);
+    return;
   }
   const T cs2 = T(1.0 / 3.0);
   gx = rdiv(gx, cs2);

@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(NT, run_blocks(sizeof(typename Store<S>::T))) 
   // own nodes: the totals f_a (FP64: replaced by their moments and s_v), rho_R, rho_B, 1 / rho
   T* const sf = carve<T>(sp, size_t(12) * NO);
   T* const sw = carve<T>(sp, size_t(8) * tl.nw);       // wall nodes: the candidates of Eq. 34; gradient, n
-  T* const sden = carve<T>(sp, tl.nv + tl.nvn);        // Eq. 29 weights of the virtual nodes, of rho^N and of n
+  T* const sden = carve<T>(sp, tl.nv + tl.nvn);        // mean_factor of the virtual nodes, of rho^N and of n
   int* const r_off = carve<int>(sp, NR);
   uint32_t* const r_tab = carve<uint32_t>(sp, NR);
   uint16_t* const r_band = carve<uint16_t>(sp, NR);
@@ -175,11 +175,11 @@ __global__ void __launch_bounds__(NT, run_blocks(sizeof(typename Store<S>::T))) 
   }
   for (int i = t; i < tl.nv; i += NT) {
     v_sten[i] = A.v_sten[tl.v0 + i];
-    sden[i] = virtual_weight<T>(v_sten[i].i);
+    sden[i] = mean_factor(virtual_weight<T>(v_sten[i].i));
   }
   for (int i = t; i < tl.nvn; i += NT) {
     vn[i] = A.vn[tl.vn0 + i];
-    sden[tl.nv + i] = virtual_weight<T>(vn[i].w);
+    sden[tl.nv + i] = mean_factor(virtual_weight<T>(vn[i].w));
   }
   for (int i = t; i < tl.ncopy; i += NT) copies[i] = A.copies[tl.copy0 + i];
   __syncthreads();
@@ -234,7 +234,8 @@ __global__ void __launch_bounds__(NT, run_blocks(sizeof(typename Store<S>::T))) 
       }
       if (tab & kSlotEdge) zou_he<T>(tab & kSlotOutlet ? nx - 1 : 0, nx, s_u[tab >> kSlotRow], C.rho_out, fr, fb);
       T rhoR, rhoB, irho;
-      srn[i] = indicator(fr, fb, rhoR, rhoB, irho);
+      const T rn = indicator(fr, fb, rhoR, rhoB, irho);
+      srn[i] = rn;
       const uint32_t own = tab & 0xFFFFu;
       if (own != 0xFFFFu) {
 #pragma unroll
@@ -244,7 +245,10 @@ __global__ void __launch_bounds__(NT, run_blocks(sizeof(typename Store<S>::T))) 
         sf[11 * NO + own] = irho;
       }
       const uint32_t band = r_band[i];
-      if (band != kNone) swv[band] = rdiv(rsub(rhoR, rhoB), radd(rhoR, rhoB));   // Eq. 12 as k_wall rounds it
+      if (band != kNone) {   // as k_wall rounds it
+        if constexpr (sizeof(T) == 8) swv[band] = rn;
+        else swv[band] = rdiv(rsub(rhoR, rhoB), radd(rhoR, rhoB));
+      }
     }
     __syncthreads();
     // ---- gradient and n of the bulk nodes of tile + 1, beside the wall chain (Eq. 28-36)
@@ -270,6 +274,7 @@ __global__ void __launch_bounds__(NT, run_blocks(sizeof(typename Store<S>::T))) 
           const int c = ((e >> 24) + 2) * CW + ((e >> 16) & 0xFFu) + 2;
           Moments<T> m;
           m.of(f);
+          relax_rest(m, radd(sf[9 * NO + i], sf[10 * NO + i]), K);
           sf[i] = m.e;
           sf[NO + i] = m.eps;
           sf[2 * NO + i] = m.jx;
@@ -306,12 +311,11 @@ __global__ void __launch_bounds__(NT, run_blocks(sizeof(typename Store<S>::T))) 
       for (int j = w; j < 2 * tl.nvn; j += kWallTeam) {
         const RunVirtN& q = vn[j >> 1];
         const T* const wn = sw + (6 + (j & 1)) * tl.nw;
-        const T den = sden[tl.nv + (j >> 1)];
         T v = T(0);
 #pragma unroll
         for (int b = 1; b < 9; ++b)
           if (q.w[b - 1] != kWallNone) v = fma_(wgt<T>(b), wn[q.w[b - 1]], v);
-        (j & 1 ? sny : snx)[q.pos] = den > T(0) ? rdiv(v, den) : T(0);
+        (j & 1 ? sny : snx)[q.pos] = mean_of(v, sden[tl.nv + (j >> 1)]);
       }
     }
     __syncthreads();
