@@ -1111,8 +1111,7 @@ cudaError_t launch_reverse(const RevRunT<R>& P, int ntiles, int threads, cudaStr
 }
 template <typename R>
 cudaError_t reverse_blocks(int threads, int* per_sm) {
-  const cudaError_t e =
-      cudaFuncSetAttribute(k_reverse<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(reverse_smem<R>(threads)));
+  const cudaError_t e = allow_max_smem(k_reverse<R>);
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_reverse<R>, threads, reverse_smem<R>(threads));
 }

@@ -51,6 +51,19 @@ cudaError_t launch_sr_tick(uint32_t* epoch, cudaStream_t st);
 // before any launch or graph capture of that precision.
 cudaError_t prepare_kernels(int prec);
 
+// Lets a kernel's launches take all the dynamic shared memory a block can have on the device.
+template <typename K>
+inline cudaError_t allow_max_smem(K* k) {
+  int dev = 0, most = 0;
+  cudaFuncAttributes a{};
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, most - int(a.sharedSizeBytes));
+  return e;
+}
+
 // ---- the resident step kernel (lbcg_run.cu)
 constexpr int kRunFlagStride = 32;   // unsigned ints between the tiles' progress words (128 bytes)
 constexpr int kReplaySteps = 32;     // steps of one graph replay of the launch-per-step schedule

@@ -413,7 +413,9 @@ cudaError_t launch(const RunArgs& a, int ntiles, int threads, size_t smem, cudaS
 
 template <typename K>
 cudaError_t prepare_k(K* k, int threads, size_t smem, int* per_sm) {
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  // the attribute belongs to the kernel, not to a handle: always the most a block can have, so
+  // that a later handle with smaller tiles takes nothing from an earlier one
+  cudaError_t e = allow_max_smem(k);
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k, threads, smem);
   return e;
 }

@@ -111,3 +111,28 @@ def test_long_call_and_configuration_sizes():
         assert np.array_equal(A.populations(), B.populations()), g.name
         A.close()
         B.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32", "fp16"])
+def test_handles_of_several_sizes_step_in_turn(prec):
+    # the kernel's shared-memory limit is the process's: a handle with larger tiles still steps after
+    # handles with smaller ones were created, and the other way round
+    from paper_1707_00198_gb300.lbcg import Lattice
+    sizes = [(600, 100), (40, 20), (300, 60)]
+    gs = [I.displacement_channel(W=w, L=l, x_I=15.0, seed=l) for l, w in sizes]
+    p = I.fingering_params(5.0, 0.1, 60.0)
+    hs = [Lattice(g, p, prec) for g in gs]
+    for L in hs:
+        L.set_tile(8)
+    for _ in range(2):
+        for L in hs:
+            L.step(40)
+    hs[0].autotune(4)
+    for g, L in zip(gs, hs):
+        one = Lattice(g, p, prec)
+        one.set_tile(8)
+        one.step(40)
+        one.step(40)
+        assert np.array_equal(L.populations(), one.populations()), (g.name, prec)
+        one.close()
+        L.close()
