@@ -488,6 +488,9 @@ lbcg_status plan_run(lbcg_handle* h) {
     return fail(LBCG_E_NOMEM, "cannot allocate the plan of the resident kernel");
   CK(h, cudaMemcpy(h->d_run, host.data(), host.size(), cudaMemcpyHostToDevice));
   CK(h, cudaMemset(h->d_progress, 0, pb));
+  // both may still be under way when they return, and the handle's stream need not wait for the
+  // legacy stream they run on
+  CK(h, cudaStreamSynchronize(cudaStreamLegacy));
   RunArgs a{};
   a.lats = h->d_lats;
   a.tiles = reinterpret_cast<const RunTile*>(h->d_run + at[0]);
@@ -865,7 +868,7 @@ lbcg_status lbcg_create_batch(int32_t n, const lbcg_geometry* geoms, const lbcg_
     // default schedule: the y-sweep when its strips give every SM a block, else tiles
     // (FP64 arithmetic is slow per SM, so FP64 takes the smallest tiles, i.e. the most blocks).
     // FP64 lattices that the resident kernel holds take the tiles in any case: 2000 x 102,
-    // 248 us per step swept, 123 resident.
+    // 248 us per step swept, 111 resident.
     if (s == LBCG_OK && h->nstrips >= kSMs && precision == LBCG_FP64) s = plan_run(h);
     if (s == LBCG_OK && (h->nstrips < kSMs || (precision == LBCG_FP64 && h->run_tiles > 0))) {
       h->sweep = 0;
