@@ -484,8 +484,14 @@ lbcg_status plan_run(lbcg_handle* h) {
   for (size_t i = 0; i < parts.size(); ++i)
     if (parts[i].second) memcpy(host.data() + at[i], parts[i].first, parts[i].second);
   const size_t pb = p.tiles.size() * kRunFlagStride * sizeof(unsigned);
-  if (!dev_alloc(h, (void**)&h->d_run, host.size()) || !dev_alloc(h, (void**)&h->d_progress, pb))
-    return fail(LBCG_E_NOMEM, "cannot allocate the plan of the resident kernel");
+  // without memory for the plan the handle keeps one launch per kernel and step
+  if (!dev_alloc(h, (void**)&h->d_run, host.size()) || !dev_alloc(h, (void**)&h->d_progress, pb)) {
+    cudaGetLastError();
+    dev_free(h, h->d_run);
+    h->d_run = nullptr;
+    h->d_progress = nullptr;
+    return LBCG_OK;
+  }
   CK(h, cudaMemcpy(h->d_run, host.data(), host.size(), cudaMemcpyHostToDevice));
   CK(h, cudaMemset(h->d_progress, 0, pb));
   // both may still be under way when they return, and the handle's stream need not wait for the

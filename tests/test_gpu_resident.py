@@ -136,3 +136,81 @@ def test_handles_of_several_sizes_step_in_turn(prec):
         assert np.array_equal(L.populations(), one.populations()), (g.name, prec)
         one.close()
         L.close()
+
+
+def test_handles_on_their_own_streams_run_at_once():
+    # four handles, each with a stream of its own, stepped from four threads: cooperative launches of
+    # one process beside each other give the bits of one after another
+    import threading
+    from paper_1707_00198_gb300.lbcg import Lattice
+    cases = [("fp32", I.config_fingering(M=5.0)), ("fp32", I.config_static_droplet()),
+             ("fp64", I.config_static_droplet()), ("fp16", I.config_capillary())]
+    one = []
+    for prec, (g, p) in cases:
+        L = Lattice(g, p, prec)
+        for _ in range(4):
+            L.step(100)
+        one.append(L.populations())
+        L.close()
+    hs = [Lattice(g, p, prec) for prec, (g, p) in cases]
+
+    def work(L):
+        for _ in range(4):
+            L.step(100)
+
+    ts = [threading.Thread(target=work, args=(L,)) for L in hs]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    for L, want, (prec, (g, _)) in zip(hs, one, cases):
+        assert np.array_equal(L.populations(), want), (prec, g.name)
+        L.close()
+
+
+def test_allocator_that_refuses_one_block():
+    # every allocation of a handle refused in turn: an error, and nothing kept, or for the two of the
+    # resident kernel's plan (an extra) a handle that steps one launch per kernel and step
+    import torch
+    from paper_1707_00198_gb300 import lbcg
+    g, p = I.config_static_droplet()
+    held, calls = {}, [0, -1]
+
+    def alloc(nbytes, stream):
+        calls[0] += 1
+        if calls[0] - 1 == calls[1]:
+            return 0
+        t = torch.empty(nbytes + 256, dtype=torch.uint8, device="cuda")
+        q = (t.data_ptr() + 255) & ~255
+        held[q] = t
+        return q
+
+    def release(q, stream):
+        torch.cuda.synchronize()
+        held.pop(q)
+
+    lbcg.lbcg_set_allocator(alloc, release)
+    try:
+        L = lbcg.Lattice(g, p, "fp32")
+        total = calls[0]
+        L.step(40)
+        assert L.step_launches == 1
+        want = L.populations()
+        L.close()
+        launched = 0
+        for k in range(total):
+            calls[:] = [0, k]
+            try:
+                L = lbcg.Lattice(g, p, "fp32")
+            except lbcg.LBCGError as e:
+                assert e.status == 8 and not held
+                continue
+            launched += 1
+            L.step(40)
+            assert L.step_launches > 40
+            assert np.array_equal(L.populations(), want)
+            L.close()
+        assert launched == 2
+    finally:
+        lbcg.lbcg_set_allocator()
+    assert not held
