@@ -733,8 +733,9 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_rho(AdjDevT<R> A) {
 // 400 x 42, FP32 forward and reverse, us per step of the whole gradient (800 steps): launched
 // stages 33.8 (with the resident forward steps), resident with the launched stages' bodies 44.7,
 // with tiles in shared memory 26.1, with the node's own values there too 24.0, beside the
-// recompute 22.0; FP64 reverse of an FP32 forward 85 -> 57, FP64 both 124 -> 89.  What bounds it: three
-// waits per reverse step (about 4,000 cycles each with the fence before them) and the latency of
+// recompute 22.0; FP64 reverse of an FP32 forward 85 -> 57, FP64 both 124 -> 89; without a __threadfence before the
+// releases 21.9 -> 20.2, 56.7 -> 55.4 and 81.8 -> 81.1.  What bounds it: three
+// waits per reverse step (about 3,300 cycles each with the release before them) and the latency of
 // the stages (6,100, 5,300 and 4,100 cycles for one or two warps per scheduler).
 __device__ __forceinline__ unsigned flag_acquire(const unsigned* p) {
   unsigned v;
@@ -847,10 +848,7 @@ __global__ void __launch_bounds__(kRevMaxThreads, sizeof(R) == 4 ? 2 : 1) k_reve
   auto arrive = [&] {
     __syncthreads();
     ++phase;
-    if (threadIdx.x == 0) {
-      __threadfence();
-      flag_release(P.progress + blockIdx.x * kRunFlagStride, phase);
-    }
+    if (threadIdx.x == 0) flag_release(P.progress + blockIdx.x * kRunFlagStride, phase);
   };
   auto wait = [&]() -> bool {
     bool lost = false;

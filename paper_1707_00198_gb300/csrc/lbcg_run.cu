@@ -16,14 +16,16 @@
 // the two without a change of bits.
 //
 // What bounds it: on the smallest lattices the chain of one step (a flag's round trip through
-// L2, about 4000 cycles with the fence before it, then the loads, the wall chain and the collision
+// L2, about 3300 cycles with the release of the stores before it, then the loads, the wall chain and the collision
 // of one pass); on the larger ones instruction issue; in FP64 the FP64 pipe.  Per step, launch per
 // kernel -> resident: 100 x 50 FP64 26.5 -> 12.6 us, 1200 x 80 FP64 72 -> 35.5, FP32 10.5 -> 5.3,
 // 2000 x 102 FP32 17.3 -> 9.4, FP16 18.6 -> 9.3, 8 x 630 x 60 FP32 with Poiseuille inlets 36 -> 12.8
 // (18.4 with the inlet profile evaluated, in FP64, at every read of an edge node).  FP32 arithmetic:
 // two blocks of 256 threads per SM, whose waits overlap each other's work, against one of 512:
 // 2000 x 102 FP32 9.4 -> 9.1, FP16 9.3 -> 8.7, 8 x 630 x 60 12.8 -> 11.8; with the push offsets of
-// bulk nodes apart from those of wall nodes 8.7, 8.5 and 11.3.
+// bulk nodes apart from those of wall nodes 8.7, 8.5 and 11.3.  FP64 with one reciprocal square root
+// per node in the wall chain (lbcg_node.cuh): 100 x 50 12.6 -> 10.0 us, 1200 x 80 35.5 -> 34.6,
+// 2000 x 102 123 -> 111.
 #include "lbcg_internal.h"
 #include "lbcg_node.cuh"
 
@@ -388,7 +390,9 @@ __global__ void __launch_bounds__(NT, run_blocks(sizeof(typename Store<S>::T))) 
     }
     __syncthreads();
     if (t == 0) {
-      __threadfence();
+      // the release at GPU scope orders the whole block's stores, which the barrier puts before it;
+      // a __threadfence ahead of it was a second trip to L2: 100 x 50 FP32 3.61 -> 3.28 us per step,
+      // 1200 x 80 FP32 5.66 -> 5.38, 2000 x 102 FP32 9.0 -> 8.6, FP16 8.6 -> 8.3
       store_release(A.progress + blockIdx.x * kRunFlagStride, A.base + unsigned(s) + 1u);
     }
   }
