@@ -28,7 +28,7 @@ __global__ void __launch_bounds__(256) k_noalloc_partial(const double* __restric
   lbcg::obs_block_partials(fields, fields + nn, fields + 2 * nn, fields + 3 * nn, mask, nx, ny, nx, partials);
 }
 
-__global__ void __launch_bounds__(32) k_noalloc_final(const double* __restrict__ partials, double* __restrict__ out) {
+__global__ void __launch_bounds__(lbcg::kObsThreads) k_noalloc_final(const double* __restrict__ partials, double* __restrict__ out) {
   lbcg::obs_final(partials, kObsBlocks, out);
 }
 
@@ -58,7 +58,7 @@ extern "C" lbcg_status lbcg_field_moments_noalloc(const double* fields, const ui
   if (e != cudaSuccess) return noalloc_fail(LBCG_E_CUDA, cudaGetErrorString(e));
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   k_noalloc_partial<<<kObsBlocks, 256, 0, st>>>(fields, mask, nx, ny, static_cast<double*>(scratch));
-  k_noalloc_final<<<1, 32, 0, st>>>(static_cast<const double*>(scratch), out);
+  k_noalloc_final<<<1, lbcg::kObsThreads, 0, st>>>(static_cast<const double*>(scratch), out);
   e = cudaGetLastError();
   if (e != cudaSuccess) return noalloc_fail(LBCG_E_CUDA, cudaGetErrorString(e));
   return LBCG_OK;

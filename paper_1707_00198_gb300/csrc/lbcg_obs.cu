@@ -16,17 +16,18 @@ __global__ void __launch_bounds__(256) k_obs_partial(const LatDev* __restrict__ 
                      macro + 3 * node_total + L.node_off, flags + L.node_off, L.nx, L.ny, L.pitch, partials);
 }
 
-__global__ void __launch_bounds__(32) k_obs_final(const double* __restrict__ partials, int nblocks,
-                                                  double* __restrict__ out) {
-  obs_final(partials, nblocks, out);
-}
-
-// First rho^N >= 0 -> rho^N < 0 change along a row (block 0: mean of rows r0, r1 -> the finger
-// tip; blocks 1, 2: rows c0, c1 -> the contact line); -1 if none.
-__global__ void __launch_bounds__(256) k_obs_rows(const LatDev* __restrict__ lats, int lat,
-                                                  const double* __restrict__ macro, long long node_total,
-                                                  const uint8_t* __restrict__ flags, int r0, int r1, int c0, int c1,
-                                                  double* __restrict__ out) {
+// Block kObsRows: the rows of partials combined.  Blocks below it: the first rho^N >= 0 -> rho^N < 0
+// change along a row (block 0: mean of rows r0, r1 -> the finger tip; blocks 1, 2: rows c0, c1 -> the
+// contact line); -1 if none.
+__global__ void __launch_bounds__(kObsThreads) k_obs_final(const double* __restrict__ partials, int nblocks,
+                                                           const LatDev* __restrict__ lats, int lat,
+                                                           const double* __restrict__ macro, long long node_total,
+                                                           const uint8_t* __restrict__ flags, int r0, int r1, int c0,
+                                                           int c1, double* __restrict__ out) {
+  if (blockIdx.x == kObsRows) {
+    obs_final(partials, nblocks, out);
+    return;
+  }
   const LatDev& L = lats[lat];
   const int ra = blockIdx.x == 0 ? r0 : (blockIdx.x == 1 ? c0 : c1);
   const int rb = blockIdx.x == 0 ? r1 : ra;
@@ -48,7 +49,7 @@ __global__ void __launch_bounds__(256) k_obs_rows(const LatDev* __restrict__ lat
       }
     }
   }
-  __shared__ int sb[8];
+  __shared__ int sb[kObsThreads / 32];
   for (int o = 16; o > 0; o >>= 1) best = min(best, __shfl_down_sync(0xffffffffu, best, o));
   if ((threadIdx.x & 31) == 0) sb[threadIdx.x >> 5] = best;
   __syncthreads();
@@ -70,8 +71,8 @@ cudaError_t launch_observables(const LatDev* lats, int lat, int nx, int ny, cons
   (void)nx;
   (void)ny;
   k_obs_partial<<<kObsBlocks, 256, 0, st>>>(lats, lat, macro, node_total, flags, partials);
-  k_obs_final<<<1, 32, 0, st>>>(partials, kObsBlocks, out);
-  k_obs_rows<<<kObsRows, 256, 0, st>>>(lats, lat, macro, node_total, flags, tip0, tip1, cl0, cl1, out);
+  k_obs_final<<<kObsRows + 1, kObsThreads, 0, st>>>(partials, kObsBlocks, lats, lat, macro, node_total, flags, tip0,
+                                                    tip1, cl0, cl1, out);
   return cudaGetLastError();
 }
 
@@ -144,16 +145,11 @@ __global__ void __launch_bounds__(256) k_diag_partial(const LatDev* __restrict__
   }
 }
 
-__global__ void __launch_bounds__(32) k_diag_final(const double* __restrict__ partials, int nblocks,
-                                                   double* __restrict__ out) {
-  const int j = threadIdx.x;
-  if (j >= kDiagQ) return;
-  double v = partials[j];
-  for (int b = 1; b < nblocks; ++b) {
-    const double w = partials[b * kDiagQ + j];
-    v = diag_max_slot(j) ? fmax(v, w) : v + w;
-  }
-  out[j] = v;
+__global__ void __launch_bounds__(kDiagQ * 32) k_diag_final(const double* __restrict__ partials, int nblocks,
+                                                            double* __restrict__ out) {
+  const int j = threadIdx.x >> 5;
+  const double v = obs_rows(partials, nblocks, kDiagQ, j, diag_max_slot(j));
+  if ((threadIdx.x & 31) == 0) out[j] = v;
 }
 
 }  // namespace
@@ -163,7 +159,7 @@ cudaError_t launch_diagnostics(const LatDev* lats, int lat, const double* macro,
                                double* partials, double* out, cudaStream_t st) {
   k_diag_partial<<<kObsBlocks, 256, 0, st>>>(lats, lat, macro, node_total, flags, usnap, have_snap ? 1 : 0, cx, cy,
                                              r * r, partials);
-  k_diag_final<<<1, 32, 0, st>>>(partials, kObsBlocks, out);
+  k_diag_final<<<1, kDiagQ * 32, 0, st>>>(partials, kObsBlocks, out);
   return cudaGetLastError();
 }
 
