@@ -168,12 +168,7 @@ __global__ void __launch_bounds__(kWallThreads, sizeof(S) == 8 ? 3 : 5) k_wall(c
           zou_he<T>(x, sL.nx, inlet_u<T>(sL, y), T(sL.rho_out), fr[v], fb[v]);
         }
         T rR, rB;
-        if constexpr (sizeof(T) == 8) {
-          T irho;
-          val[i] = indicator(fr[v], fb[v], rR, rB, irho);
-        } else {
-          val[i] = colour_indicator(fr[v], fb[v], rR, rB);
-        }
+        val[i] = colour_indicator(fr[v], fb[v], rR, rB);
       }
     }
   }
@@ -191,7 +186,7 @@ __global__ void __launch_bounds__(kWallThreads, sizeof(S) == 8 ? 3 : 5) k_wall(c
           num = radd(num, rmul(wgt<T>(b), val[q.i[b - 1]]));
           den = radd(den, wgt<T>(b));
         }
-      v = mean_of(num, mean_factor(den));
+      v = rdiv(num, den);
     }
     val[G.nband + j] = v;
   }

@@ -325,7 +325,8 @@ struct Recolour {
 };
 
 // Virtual value of Eq. 29 on an outermost solid node: the weighted mean of `val` over its fluid
-// neighbours (local indices q, kWallNone where the neighbour is solid); factor: mean_factor(virtual_weight(q))
+// neighbours (local indices q, kWallNone where the neighbour is solid); den: virtual_weight(q).  Divided in
+// FP64 too: equal neighbours give equal values, and what Eq. 36 picks between can hang on the last bit.
 template <typename T>
 __device__ __forceinline__ T virtual_weight(const uint16_t q[8]) {
   T den = T(0);
@@ -334,7 +335,7 @@ __device__ __forceinline__ T virtual_weight(const uint16_t q[8]) {
     if (q[b - 1] != kWallNone) den = radd(den, wgt<T>(b));
   return den;
 }
-// What a sum over the fluid neighbours is divided by (FP32) or multiplied with (FP64: the
+// What a sum of n over the fluid neighbours is divided by (FP32) or multiplied with (FP64: the
 // reciprocal, 1 operation instead of 9), from the weight
 template <typename T>
 __device__ __forceinline__ T mean_factor(T den) {
@@ -347,12 +348,12 @@ __device__ __forceinline__ T mean_of(T num, T factor) {
   else return rdiv(num, factor);
 }
 template <typename T>
-__device__ __forceinline__ T virtual_value(const WallSten& q, const T* val, T factor) {
+__device__ __forceinline__ T virtual_value(const WallSten& q, const T* val, T den) {
   T num = T(0);
 #pragma unroll
   for (int b = 1; b < 9; ++b)
     if (q.i[b - 1] != kWallNone) num = radd(num, rmul(wgt<T>(b), val[q.i[b - 1]]));
-  return mean_of(num, factor);
+  return rdiv(num, den);
 }
 
 // The two candidates of Eq. 34 on an outermost fluid node (rotations by +theta and -theta)
@@ -362,6 +363,15 @@ __device__ __forceinline__ void wall_candidates(T nsx, T nsy, T c, T s, T& f1x, 
   f1y = radd(rmul(nsx, s), rmul(nsy, c));
   f2x = radd(rmul(nsx, c), rmul(nsy, s));
   f2y = radd(rmul(-nsx, s), rmul(nsy, c));
+}
+
+// FP64: whether two squared distances of Eq. 35 (at most 4) are equal but for their rounding and that of
+// the steps before them, a few 1e-15.  The pick of Eq. 36 then follows the operations as the equations
+// have them (square roots, divisions), in the oracle's order: next to a wall at 90 degrees a gradient
+// along the wall's normal is such a tie, and n would point along the wall one way or the other.
+template <typename T>
+__device__ __forceinline__ bool near_tie(T d1, T d2) {
+  return fabs(rsub(d1, d2)) <= T(1e-13);
 }
 
 // wall_normal (below) by two neighbouring lanes, r = 0 for x and r = 1 for y: each takes its
@@ -380,6 +390,7 @@ __device__ __forceinline__ void wall_normal_pair(T eps, int wetting, T f1, T f2,
   g = radd(g, r ? v6 : -v6);
   g = radd(g, -v(7));
   g = radd(g, r ? -v8 : v8);
+  [[maybe_unused]] const T sum = g;
   if constexpr (sizeof(T) == 8) g = rmul(g, T(3));
   else g = rdiv(g, T(1.0 / 3.0));
   auto other = [](T x) { return __shfl_xor_sync(0xFFFFFFFFu, x, 1); };
@@ -396,7 +407,16 @@ __device__ __forceinline__ void wall_normal_pair(T eps, int wetting, T f1, T f2,
     }
     const T a1 = rsub(cx, r ? eo : es), b1 = rsub(cy, r ? es : eo);
     const T d = radd(rmul(a1, a1), rmul(b1, b1)), od = other(d);
-    const T nf = (r ? od <= d : d <= od) ? f1 : f2;
+    bool one = r ? od <= d : d <= od;
+    const bool close = near_tie(d, od);
+    if (__any_sync(0xFFFFFFFFu, close)) {
+      const T ge = rdiv(sum, T(1.0 / 3.0)), gge = rmul(ge, ge), mage = rsqrt_(radd(gge, other(gge)));
+      const T ese = rdiv(ge, on ? mage : T(1)), eoe = other(ese);
+      const T ae = rsub(cx, r ? eoe : ese), be = rsub(cy, r ? ese : eoe);
+      const T de = rsqrt_(radd(rmul(ae, ae), rmul(be, be))), ode = other(de);
+      if (close) one = r ? ode <= de : de <= ode;
+    }
+    const T nf = one ? f1 : f2;
     if (on) {
       cg = rmul(mag, nf);
       n = nf;
@@ -426,8 +446,8 @@ __device__ __forceinline__ void wall_normal_pair(T eps, int wetting, T f1, T f2,
 // contact-angle correction of Eq. 30-36 -> corrected gradient and unit normal.  The sums run
 // in the oracle's order (directions 1..8, products w*phi then sign), so that a gradient exactly
 // along the wall's normal makes Eq. 35-36 an exact tie.  FP64 takes one reciprocal square root in
-// place of three square roots and seven divisions: it compares the squared distances (equal
-// whenever the distances of an exact tie are) and takes n = n_f (28 operations against 78).
+// place of three square roots and seven divisions: it compares the squared distances (near a tie
+// the distances themselves) and takes n = n_f (30 operations against 78).
 template <typename T>
 __device__ __forceinline__ void wall_normal(T eps, int wetting, T nsx, T nsy, T c, T s, const WallSten& q, const T* val,
                                             T& cgx, T& cgy, T& nx, T& ny) {
@@ -441,6 +461,7 @@ __device__ __forceinline__ void wall_normal(T eps, int wetting, T nsx, T nsy, T 
     if (ey(a) == -1) gy = radd(gy, -tt);
   }
   if constexpr (sizeof(T) == 8) {
+    const T sx = gx, sy = gy;
     gx = rmul(gx, T(3));
     gy = rmul(gy, T(3));
     const T m2 = radd(rmul(gx, gx), rmul(gy, gy)), inv = rsqrt(m2), mag = rmul(m2, inv);
@@ -457,7 +478,15 @@ __device__ __forceinline__ void wall_normal(T eps, int wetting, T nsx, T nsy, T 
     T f1x, f1y, f2x, f2y;
     wall_candidates<T>(nsx, nsy, c, s, f1x, f1y, f2x, f2y);
     const T a1 = rsub(f1x, esx), b1 = rsub(f1y, esy), a2 = rsub(f2x, esx), b2 = rsub(f2y, esy);
-    const bool one = radd(rmul(a1, a1), rmul(b1, b1)) <= radd(rmul(a2, a2), rmul(b2, b2));
+    const T d1 = radd(rmul(a1, a1), rmul(b1, b1)), d2 = radd(rmul(a2, a2), rmul(b2, b2));
+    bool one = d1 <= d2;
+    if (near_tie(d1, d2)) {
+      const T gex = rdiv(sx, T(1.0 / 3.0)), gey = rdiv(sy, T(1.0 / 3.0));
+      const T mage = rsqrt_(radd(rmul(gex, gex), rmul(gey, gey)));
+      const T ex_ = rdiv(gex, mage), ey_ = rdiv(gey, mage);
+      const T p1 = rsub(f1x, ex_), q1 = rsub(f1y, ey_), p2 = rsub(f2x, ex_), q2 = rsub(f2y, ey_);
+      one = rsqrt_(radd(rmul(p1, p1), rmul(q1, q1))) <= rsqrt_(radd(rmul(p2, p2), rmul(q2, q2)));
+    }
     nx = one ? f1x : f2x;
     ny = one ? f1y : f2y;
     cgx = rmul(mag, nx);

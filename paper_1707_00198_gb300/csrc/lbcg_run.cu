@@ -24,8 +24,9 @@
 // two blocks of 256 threads per SM, whose waits overlap each other's work, against one of 512:
 // 2000 x 102 FP32 9.4 -> 9.1, FP16 9.3 -> 8.7, 8 x 630 x 60 12.8 -> 11.8; with the push offsets of
 // bulk nodes apart from those of wall nodes 8.7, 8.5 and 11.3.  FP64 with one reciprocal square root
-// per node in the wall chain (lbcg_node.cuh): 100 x 50 12.6 -> 10.0 us, 1200 x 80 35.5 -> 34.6,
-// 2000 x 102 123 -> 111.
+// per node in the wall chain (lbcg_node.cuh): 100 x 50 12.6 -> 10.5 us, 1200 x 80 35.5 -> 35.2,
+// 2000 x 102 123 -> 111 (9.9, 34.6 and 111 with the divisions of rho^N and of Eq. 29 also reciprocals, which
+// decides near ties of Eq. 36 otherwise than the equations' own operations).
 #include "lbcg_internal.h"
 #include "lbcg_node.cuh"
 
@@ -94,7 +95,7 @@ __global__ void __launch_bounds__(NT, run_blocks(sizeof(typename Store<S>::T))) 
   // own nodes: the totals f_a (FP64: replaced by their moments and s_v), rho_R, rho_B, 1 / rho
   T* const sf = carve<T>(sp, size_t(12) * NO);
   T* const sw = carve<T>(sp, size_t(8) * tl.nw);       // wall nodes: the candidates of Eq. 34; gradient, n
-  T* const sden = carve<T>(sp, tl.nv + tl.nvn);        // mean_factor of the virtual nodes, of rho^N and of n
+  T* const sden = carve<T>(sp, tl.nv + tl.nvn);        // virtual nodes: the weight (of rho^N), mean_factor (of n)
   int* const r_off = carve<int>(sp, NR);
   uint32_t* const r_tab = carve<uint32_t>(sp, NR);
   uint16_t* const r_band = carve<uint16_t>(sp, NR);
@@ -177,7 +178,7 @@ __global__ void __launch_bounds__(NT, run_blocks(sizeof(typename Store<S>::T))) 
   }
   for (int i = t; i < tl.nv; i += NT) {
     v_sten[i] = A.v_sten[tl.v0 + i];
-    sden[i] = mean_factor(virtual_weight<T>(v_sten[i].i));
+    sden[i] = virtual_weight<T>(v_sten[i].i);
   }
   for (int i = t; i < tl.nvn; i += NT) {
     vn[i] = A.vn[tl.vn0 + i];
@@ -236,8 +237,7 @@ __global__ void __launch_bounds__(NT, run_blocks(sizeof(typename Store<S>::T))) 
       }
       if (tab & kSlotEdge) zou_he<T>(tab & kSlotOutlet ? nx - 1 : 0, nx, s_u[tab >> kSlotRow], C.rho_out, fr, fb);
       T rhoR, rhoB, irho;
-      const T rn = indicator(fr, fb, rhoR, rhoB, irho);
-      srn[i] = rn;
+      srn[i] = indicator(fr, fb, rhoR, rhoB, irho);
       const uint32_t own = tab & 0xFFFFu;
       if (own != 0xFFFFu) {
 #pragma unroll
@@ -247,10 +247,7 @@ __global__ void __launch_bounds__(NT, run_blocks(sizeof(typename Store<S>::T))) 
         sf[11 * NO + own] = irho;
       }
       const uint32_t band = r_band[i];
-      if (band != kNone) {   // as k_wall rounds it
-        if constexpr (sizeof(T) == 8) swv[band] = rn;
-        else swv[band] = rdiv(rsub(rhoR, rhoB), radd(rhoR, rhoB));
-      }
+      if (band != kNone) swv[band] = rdiv(rsub(rhoR, rhoB), radd(rhoR, rhoB));   // as k_wall rounds it
     }
     __syncthreads();
     // ---- gradient and n of the bulk nodes of tile + 1, beside the wall chain (Eq. 28-36)

@@ -214,3 +214,29 @@ def test_allocator_that_refuses_one_block():
     finally:
         lbcg.lbcg_set_allocator()
     assert not held
+
+
+@pytest.mark.parametrize("schedule", ["tiles", "sweep"])
+def test_gradient_along_the_walls_normal_at_90_degrees(schedule):
+    # Eq. 36 picks between two normals along the wall; a gradient along the wall's own normal (one
+    # mixed node in pure fluid beside the wall) leaves them equally near but for rounding, so that every
+    # operation of the chain before has to be the oracle's
+    from oracle import lbcg_oracle as O
+    from paper_1707_00198_gb300.lbcg import Lattice
+    rng = np.random.default_rng(3)
+    g = I.flat_wall_droplet(120, 90, R=20.0, closed_x=True)
+    rho_n = np.full((90, 120), -1.0)
+    for k in range(4, 86, 6):
+        rho_n[k, 1] = rho_n[k, 118] = -1.0 + 1e-3 * rng.random()
+    for k in range(6, 114, 6):
+        rho_n[1, k] = rho_n[88, k] = -1.0 + 1e-3 * rng.random()
+    g = dataclasses.replace(g, rhoN0=rho_n)
+    p = I.Params(theta=math.pi / 2)
+    L = Lattice(g, p, "fp64")
+    L.set_tile(8) if schedule == "tiles" else L.set_sweep()
+    L.step(1)
+    lat = O.make_lattice(g, p.theta)
+    fR, fB = O.run(lat, p, *O.init_state(lat, g.rhoN0, p.rho0, p), 1)
+    # (a pick the other way round moves populations by 1e-5 and more; rounding by 1e-15)
+    assert float(np.abs(L.populations() - np.stack([fR.numpy(), fB.numpy()])).max()) <= 1e-12
+    L.close()
