@@ -331,7 +331,8 @@ lbcg_status lbcg_kernel_times(lbcg_handle* h, double* ms2, int64_t* steps);
  * bulk kernel), the number of kernel launches lbcg_step has enqueued on the handle since it was
  * created (each kernel node of a replayed graph counts: a batch's graph runs its lattices as
  * up to 3 parallel branches of their own launches; a cooperative launch of many steps is one,
- * with 16-bit storage two), and the number of lattice nodes (fluid and
+ * and one more where it stands for whole graph replays in 16-bit storage, whose rounding keys count
+ * them), and the number of lattice nodes (fluid and
  * solid) all lattices hold. */
 int32_t lbcg_launches_per_step(const lbcg_handle* h);
 int64_t lbcg_step_launches(const lbcg_handle* h);

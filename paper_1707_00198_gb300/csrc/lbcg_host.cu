@@ -547,7 +547,11 @@ cudaError_t enqueue_run(lbcg_handle* h, int64_t* n) {
   a.nrep = int((*n - pre) / kGraphSteps);
   h->run_base += unsigned(*n);
   cudaError_t e = launch_run(h->prec, a, h->run_tiles, h->run_threads, h->run_smem, h->stream);
-  if (e == cudaSuccess && h->prec >= 2 && a.nrep > 0) e = launch_sr_add(h->d_sr_epoch, uint32_t(a.nrep), h->stream);
+  h->step_launches += 1;
+  if (e == cudaSuccess && h->prec >= 2 && a.nrep > 0) {
+    e = launch_sr_add(h->d_sr_epoch, uint32_t(a.nrep), h->stream);
+    h->step_launches += 1;
+  }
   return e;
 }
 
@@ -966,7 +970,6 @@ lbcg_status lbcg_step(lbcg_handle* h, int64_t nsteps) {
     if (runs_resident(h, nsteps)) {
       int64_t n = nsteps;
       CK(h, enqueue_run(h, &n));
-      h->step_launches += h->prec >= 2 ? 2 : 1;
       h->cur ^= int(n & 1);
       h->step += n;
       nsteps -= n;
