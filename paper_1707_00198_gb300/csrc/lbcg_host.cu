@@ -1482,10 +1482,13 @@ lbcg_status adjoint_run(lbcg_handle* h, const lbcg_adjoint_spec* spec, lbcg_grad
   unsigned *progress2 = nullptr, *progress3 = nullptr;
   unsigned base2 = 0, base3 = 0;
   int rev_threads = 0;
-  const bool resident = !h->sweep && h->run_tiles > 0 && h->poll_limit == kPollLimit && !h->profiling;
+  bool resident = !h->sweep && h->run_tiles > 0 && h->poll_limit == kPollLimit && !h->profiling;
+  const size_t pb = size_t(h->run_tiles) * kRunFlagStride * sizeof(unsigned);
+  if (resident && (!B.get(&progress2, pb) || !B.get(&progress3, pb))) {
+    cudaGetLastError();
+    resident = false;   // without memory for the words: the launched stages
+  }
   if (resident) {
-    const size_t pb = size_t(h->run_tiles) * kRunFlagStride * sizeof(unsigned);
-    if (!B.get(&progress2, pb) || !B.get(&progress3, pb)) return fail(LBCG_E_NOMEM, "adjoint buffers");
     CK(h, cudaMemsetAsync(progress2, 0, pb, h->stream));
     CK(h, cudaMemsetAsync(progress3, 0, pb, h->stream));
     rev_threads = 2 * ((h->run_nodes + 31) / 32 * 32);
