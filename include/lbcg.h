@@ -237,10 +237,13 @@ lbcg_status lbcg_set_tile(lbcg_handle* h, int32_t ty);
  * be replaced (lbcg_set_populations, lbcg_upload_state).  lbcg_set_poll_limit sets the number
  * of polls (polls < 0 restores the default; 0 makes every wait give up at once, which tests
  * the path without any fault).  Synchronises and drops captured graphs.
- * The cooperative kernel of long calls (lbcg_step) has the other device-side wait, of a tile for
- * the tiles around it, always with the default bound and reported the same way; a handle whose
- * limit was changed launches each kernel of its steps instead. */
+ * The cooperative kernels (of long calls of lbcg_step, and of lbcg_adjoint) have the other
+ * device-side wait, of a tile for the tiles around it, with a bound of its own,
+ * lbcg_set_tile_poll_limit (the same default and the same meaning of polls), and reported the same
+ * way, by lbcg_adjoint itself where it happens there.  A handle whose lbcg_set_poll_limit was changed launches
+ * each kernel of its steps instead. */
 lbcg_status lbcg_set_poll_limit(lbcg_handle* h, int32_t polls);
+lbcg_status lbcg_set_tile_poll_limit(lbcg_handle* h, int32_t polls);
 
 /* Gradients by the discrete adjoint (reverse mode) of the step.  From the handle's current
  * state, lbcg_adjoint runs `nsteps` steps forward (storing the state every `checkpoint`

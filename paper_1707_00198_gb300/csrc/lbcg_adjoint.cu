@@ -32,6 +32,7 @@
 
 #include "../../include/lbcg.h"
 #include "lbcg_internal.h"
+#include "lbcg_wait.cuh"
 
 namespace lbcg {
 
@@ -737,15 +738,6 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_rho(AdjDevT<R> A) {
 // releases 21.9 -> 20.2, 56.7 -> 55.4 and 81.8 -> 81.1.  What bounds it: three
 // waits per reverse step (about 3,300 cycles each with the release before them) and the latency of
 // the stages (6,100, 5,300 and 4,100 cycles for one or two warps per scheduler).
-__device__ __forceinline__ unsigned flag_acquire(const unsigned* p) {
-  unsigned v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ void flag_release(unsigned* p, unsigned v) {
-  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-
 __device__ __forceinline__ void half_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 
 // (FP32: held to 128 registers, so that two blocks of 128 threads fit on an SM beside two of the
@@ -848,19 +840,12 @@ __global__ void __launch_bounds__(kRevMaxThreads, sizeof(R) == 4 ? 2 : 1) k_reve
   auto arrive = [&] {
     __syncthreads();
     ++phase;
-    if (threadIdx.x == 0) flag_release(P.progress + blockIdx.x * kRunFlagStride, phase);
+    if (threadIdx.x == 0) store_release(P.progress + blockIdx.x * kRunFlagStride, phase);
   };
   auto wait = [&]() -> bool {
     bool lost = false;
-    for (int j = threadIdx.x; j < tl.nnb; j += blockDim.x) {
-      const unsigned* p = P.progress + P.nb[tl.nb0 + j] * kRunFlagStride;
-      int polls = 0;
-      while (int(flag_acquire(p) - phase) < 0)
-        if (++polls >= P.poll_limit || ((polls & 1023) == 0 && *static_cast<volatile int*>(P.err) != 0)) {
-          lost = true;
-          break;
-        }
-    }
+    for (int j = threadIdx.x; j < tl.nnb && !lost; j += blockDim.x)
+      lost = !wait_reached(P.progress + P.nb[tl.nb0 + j] * kRunFlagStride, phase, P.poll_limit, P.err);
     if (__syncthreads_or(lost)) {
       if (threadIdx.x == 0) atomicOr(P.err, ERR_TIMEOUT);
       return false;

@@ -82,6 +82,7 @@ struct lbcg_handle {
   int scheme_b = 0;        // some lattice uses wetting scheme (b)
   int* d_err = nullptr;    // device error word (a sweep block's bounded wait ran out)
   int poll_limit = kPollLimit;   // polls of a sweep block's wait for a staged row (about a second)
+  int run_polls = kPollLimit;    // and of a resident kernel's wait for the tiles around one
   uint32_t* d_sr_epoch = nullptr;     // 16-bit storage: graph replays so far (stochastic-rounding keys)
   double* d_usnap = nullptr;          // velocity stored by lbcg_diagnostics ([2][node_total])
   std::vector<int64_t> snap_step;     // per lattice: step of that velocity, -1 = none
@@ -513,7 +514,6 @@ lbcg_status plan_run(lbcg_handle* h) {
   a.nbmask = h->d_nbmask;
   a.progress = h->d_progress;
   a.err = h->d_err;
-  a.poll_limit = kPollLimit;
   a.sr_epoch = h->d_sr_epoch;
   h->run = a;
   h->run_smem = p.smem;
@@ -541,6 +541,7 @@ cudaError_t enqueue_run(lbcg_handle* h, int64_t* n) {
   a.pool0 = static_cast<char*>(h->pool[h->cur]);
   a.pool1 = static_cast<char*>(h->pool[h->cur ^ 1]);
   a.nsteps = int(*n);
+  a.poll_limit = h->run_polls;
   a.base = h->run_base;
   a.step0 = uint32_t(h->step);
   a.pre = pre;
@@ -570,7 +571,8 @@ lbcg_status ensure_macro(lbcg_handle* h) {
 // or uploaded afterwards steps correctly again.
 lbcg_status report_device_error(lbcg_handle* h, int e) {
   if (e) {
-    if (cudaMemset(h->d_err, 0, sizeof(int)) != cudaSuccess)
+    // (on the handle's stream: before what is launched next)
+    if (cudaMemsetAsync(h->d_err, 0, sizeof(int), h->stream) != cudaSuccess)
       return cuda_fail(h, cudaGetLastError(), "clearing the device error word");
     if (e & ERR_BOUNDS)
       return fail(LBCG_E_BOUNDS, "a range check of the checked build failed in a step kernel (the access was "
@@ -1572,6 +1574,7 @@ lbcg_status adjoint_run(lbcg_handle* h, const lbcg_adjoint_spec* spec, lbcg_grad
         a.pool0 = reinterpret_cast<char*>(segs[b]) + sb * j;
         a.stride = (long long)sb;
         a.nsteps = int(std::min<int64_t>(ns - 1 - j, kRunMaxSteps));
+        a.poll_limit = h->run_polls;
         a.progress = progress2;
         a.base = base2;
         base2 += unsigned(a.nsteps);
@@ -1681,7 +1684,7 @@ lbcg_status adjoint_run(lbcg_handle* h, const lbcg_adjoint_spec* spec, lbcg_grad
       P.progress = progress3;
       P.base = base3;
       P.err = h->d_err;
-      P.poll_limit = kPollLimit;
+      P.poll_limit = h->run_polls;
       P.states = reinterpret_cast<const char*>(segs[b]);
       P.stride = (long long)sb;
       P.ns = int(ns);
@@ -1727,8 +1730,11 @@ extern "C" {
 
 lbcg_status lbcg_adjoint(lbcg_handle* h, const lbcg_adjoint_spec* spec, lbcg_grads* out) {
   Range range_("lbcg_adjoint");
-  if (spec && spec->reverse_fp32) return adjoint_run<float>(h, spec, out);
-  return adjoint_run<double>(h, spec, out);
+  const lbcg_status s = spec && spec->reverse_fp32 ? adjoint_run<float>(h, spec, out) : adjoint_run<double>(h, spec, out);
+  // a wait of the second stream may have run out too after the word was read and cleared; both
+  // streams are idle now: reported once
+  if (s == LBCG_E_TIMEOUT || s == LBCG_E_BOUNDS) CK(h, cudaMemsetAsync(h->d_err, 0, sizeof(int), h->stream));
+  return s;
 }
 
 lbcg_status lbcg_set_sweep(lbcg_handle* h, int32_t rows) {
@@ -1755,6 +1761,14 @@ lbcg_status lbcg_set_poll_limit(lbcg_handle* h, int32_t polls) {
     cudaGraphExecDestroy(h->graph);
     h->graph = nullptr;
   }
+  return LBCG_OK;
+}
+
+lbcg_status lbcg_set_tile_poll_limit(lbcg_handle* h, int32_t polls) {
+  lbcg_status s = check_handle(h);
+  if (s != LBCG_OK) return s;
+  CK(h, cudaStreamSynchronize(h->stream));
+  h->run_polls = polls < 0 ? kPollLimit : polls;
   return LBCG_OK;
 }
 
@@ -1842,6 +1856,7 @@ lbcg_status lbcg_autotune(lbcg_handle* h, int32_t probe_steps, int32_t* schedule
       a.pool0 = static_cast<char*>(h->pool[h->cur]);
       a.pool1 = static_cast<char*>(h->pool[h->cur ^ 1]);
       a.nsteps = n;
+      a.poll_limit = h->run_polls;
       for (int q = 0; q < 2 && e == cudaSuccess; ++q) {
         if (q) e = cudaEventRecord(e0, h->stream);
         a.base = h->run_base;

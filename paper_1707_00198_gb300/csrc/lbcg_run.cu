@@ -29,6 +29,7 @@
 // decides near ties of Eq. 36 otherwise than the equations' own operations).
 #include "lbcg_internal.h"
 #include "lbcg_node.cuh"
+#include "lbcg_wait.cuh"
 
 namespace lbcg {
 
@@ -48,14 +49,6 @@ __device__ __forceinline__ void load_pair_cg(const S* p, typename Store<S>::T& l
   }
 }
 
-__device__ __forceinline__ unsigned load_acquire(const unsigned* p) {
-  unsigned v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ void store_release(unsigned* p, unsigned v) {
-  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
 __device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 
 // slot table entry: own index in the low half (0xFFFF: not of the tile), and
@@ -200,18 +193,8 @@ __global__ void __launch_bounds__(NT, run_blocks(sizeof(typename Store<S>::T))) 
     bool lost = false;
     if (s > 0) {
       const unsigned want = A.base + unsigned(s);
-      for (int j = t; j < tl.nnb; j += NT) {
-        const unsigned* p = A.progress + A.nb[tl.nb0 + j] * kRunFlagStride;
-        int polls = 0;
-        while (int(load_acquire(p) - want) < 0) {
-          // bounded: after the limit, or once another block has given up, the block returns
-          // (nothing of its own is in flight)
-          if (++polls >= A.poll_limit || ((polls & 1023) == 0 && *static_cast<volatile int*>(A.err) != 0)) {
-            lost = true;
-            break;
-          }
-        }
-      }
+      for (int j = t; j < tl.nnb && !lost; j += NT)
+        lost = !wait_reached(A.progress + A.nb[tl.nb0 + j] * kRunFlagStride, want, A.poll_limit, A.err);
     }
     if (__syncthreads_or(lost)) {
       if (t == 0) atomicOr(A.err, ERR_TIMEOUT);

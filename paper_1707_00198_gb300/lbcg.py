@@ -119,6 +119,7 @@ def library():
         "lbcg_set_tile": (C.c_int, [H, C.c_int32]),
         "lbcg_set_sweep": (C.c_int, [H, C.c_int32]),
         "lbcg_set_poll_limit": (C.c_int, [H, C.c_int32]),
+        "lbcg_set_tile_poll_limit": (C.c_int, [H, C.c_int32]),
         "lbcg_set_allocator": (C.c_int, [C.POINTER(lbcg_allocator)]),
         "lbcg_profile": (C.c_int, [H, C.c_int32]),
         "lbcg_kernel_times": (C.c_int, [H, C.POINTER(C.c_double), C.POINTER(C.c_int64)]),
@@ -149,7 +150,7 @@ def exported_symbols() -> list:
             "lbcg_set_populations", "lbcg_get_fields", "lbcg_state_bytes", "lbcg_upload_state",
             "lbcg_download_state", "lbcg_set_sweep", "lbcg_set_tile", "lbcg_profile", "lbcg_kernel_times", "lbcg_launches_per_step", "lbcg_step_host", "lbcg_step_launches", "lbcg_total_nodes", "lbcg_destroy",
             "lbcg_last_error", "lbcg_field_moments_noalloc", "lbcg_adjoint", "lbcg_autotune", "lbcg_schedule", "lbcg_sweep_rows", "lbcg_diagnostics",
-            "lbcg_set_poll_limit", "lbcg_set_allocator"]
+            "lbcg_set_poll_limit", "lbcg_set_tile_poll_limit", "lbcg_set_allocator"]
 
 
 def _check(status: int):
@@ -250,6 +251,11 @@ def lbcg_set_sweep(h: int, rows: int = 0):
 def lbcg_set_poll_limit(h: int, polls: int = -1):
     """Polls of the sweep's bounded wait for a staged row (-1: the default, 0: give up at once)."""
     _check(library().lbcg_set_poll_limit(h, polls))
+
+
+def lbcg_set_tile_poll_limit(h: int, polls: int = -1):
+    """Polls of the cooperative kernels' bounded wait of a tile for the tiles around it (as above)."""
+    _check(library().lbcg_set_tile_poll_limit(h, polls))
 
 
 _allocator_keepalive = []   # every installed allocator: handles keep the one they were created with
@@ -416,6 +422,9 @@ class Lattice:
 
     def set_poll_limit(self, polls: int = -1):
         lbcg_set_poll_limit(self.h, polls)
+
+    def set_tile_poll_limit(self, polls: int = -1):
+        lbcg_set_tile_poll_limit(self.h, polls)
 
     def diagnostics(self, circle, inside_red: bool = True, lattice: int = 0) -> dict:
         return lbcg_diagnostics(self.h, lattice, circle, inside_red)
