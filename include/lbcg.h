@@ -174,7 +174,12 @@ lbcg_status lbcg_create_batch(int32_t n, const lbcg_geometry* geoms, const lbcg_
  * more, other than 32, of a handle on the tile schedule whose lattices fit on the GPU at once (one
  * tile per resident block) is launched as one cooperative kernel that takes all the steps (at
  * most 8192 per launch); other calls of 32 steps and more replay a captured CUDA graph, and short
- * ones launch each kernel.  The results do not depend on which. */
+ * ones launch each kernel.  The results do not depend on which.  Cooperative launches of several
+ * handles, each on a stream of its own, run at once where all their blocks fit on the GPU beside each
+ * other (small lattices), else one after another.  Lattices that advance together belong in one handle:
+ * eight lattices of 100 x 50 in FP32 take 0.53 us per step of each as a batch and 0.92 as eight handles
+ * at once, eight of 400 x 42 take 0.90 and 2.28.  A handle whose lbcg_set_poll_limit was changed launches
+ * each kernel, and these interleave with those of others (eight of 400 x 42: 1.50). */
 lbcg_status lbcg_step(lbcg_handle* h, int64_t nsteps);
 
 /* Measure the observables of lattice `lattice` of the current state (synchronises the

@@ -452,15 +452,24 @@ lbcg_status plan_run(lbcg_handle* h) {
   }
   // (a fluid node takes at least its 12 values and 8 bytes of tables)
   if (fluid * (long long)(12 * cs + 8) > (long long)sms * blocks * (long long)budget) return LBCG_OK;
+  // Small lattices take blocks that leave room on their SMs for those of other handles: a cooperative grid
+  // starts only once all its blocks have room, so that grids of large blocks run one after another.
+  // FP32: one tile per SM, where 128 threads take each stage of it in one pass, is as fast as two half as
+  // large (100 x 50: 3.30 us per step either way), and eight handles at once on streams of their own take 0.92 us per
+  // step of each, for 1.75.  16-bit storage keeps two (3.27 us, one 3.37).
   RunPlan p;
-  if (!build_run_plan(views, flags, h->ofb_host, blocks * sms, budget, cs, p)) return LBCG_OK;
+  const bool one = h->prec == LBCG_FP32 && fluid <= (long long)kRunSmallThreads / 2 * sms &&
+                   build_run_plan(views, flags, h->ofb_host, sms, budget, cs, p) && run_one_pass(p);
+  if (!one && !build_run_plan(views, flags, h->ofb_host, blocks * sms, budget, cs, p)) return LBCG_OK;
   for (const RunTile& t : p.tiles) {
     h->run_nodes = std::max(h->run_nodes, t.tx * t.ty);
     h->run_slots = std::max(h->run_slots, (t.tx + 4) * (t.ty + 4));
   }
-  // blocks of 128 threads where the tiles are that small: they leave registers for a kernel on
-  // another stream (the adjoint's reverse sweep beside the recompute of a segment)
-  h->run_threads = cs == 4 && h->run_nodes <= 64 ? 128 : 256;
+  // Blocks of 128 threads where the tiles are that small.  FP32: they also leave registers for a kernel on
+  // another stream (the adjoint's reverse sweep beside the recompute of a segment).  FP64: where
+  // each stage is one pass of them (100 x 50: 10.5 us per step either way; eight handles at once 6.0 us
+  // per step of each, for 10.6; with two passes 1.1 to 1.2 times the time of 256 threads).
+  h->run_threads = (cs == 4 ? h->run_nodes <= 64 : run_one_pass(p)) ? kRunSmallThreads : 256;
   int per_sm = 0;
   CK(h, prepare_run(h->prec, h->run_threads, p.smem, &per_sm));
   if ((long long)per_sm * sms < (long long)p.tiles.size()) return LBCG_OK;

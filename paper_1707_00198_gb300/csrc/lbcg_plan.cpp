@@ -16,6 +16,15 @@ size_t run_smem_bytes(const RunTile& t, size_t cs) {
          up(size_t(t.ncopy) * 4);
 }
 
+bool run_one_pass(const RunPlan& plan) {
+  for (const RunTile& t : plan.tiles) {
+    const int half = kRunSmallThreads / 2, team = t.nw > 0 ? half : kRunSmallThreads;
+    if ((t.tx + 4) * (t.ty + 4) + t.ne > kRunSmallThreads || (t.tx + 2) * (t.ty + 2) > team) return false;
+    if (t.nv > half || 2 * t.nw > half || 2 * t.nvn > half || t.ncopy > half) return false;
+  }
+  return true;
+}
+
 namespace {
 
 // fluid nodes of a lattice in any rectangle, from a summed-area table

@@ -57,6 +57,10 @@ struct RunPlan {
 // that one works while the other waits for its neighbours.  FP64: one, since the FP64 pipe is
 // the bound and a tile half as large recomputes more of its halo.
 LBCG_HD constexpr int run_blocks(size_t cs) { return cs == 4 ? 2 : 1; }
+// A block of kRunSmallThreads threads, half of them beside the tile's wall nodes where it has any.
+constexpr int kRunSmallThreads = 128;
+// Whether such blocks take every stage of every tile in one pass, so that more threads would only idle.
+bool run_one_pass(const RunPlan& plan);
 // Dynamic shared memory of a tile: `cs` bytes per value of the compute type.
 size_t run_smem_bytes(const RunTile& t, size_t cs);
 
