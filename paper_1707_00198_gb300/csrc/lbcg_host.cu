@@ -177,9 +177,13 @@ bool dev_alloc(const lbcg_handle* h, void** p, size_t bytes) {
       q = nullptr;
     }
     *p = q;
-    return q != nullptr;
+  } else if (cudaMalloc(p, bytes) != cudaSuccess) {
+    *p = nullptr;
   }
-  return cudaMalloc(p, bytes) == cudaSuccess;
+  // a refusal is the caller's to report or to do without: the runtime's last error, which the next
+  // launch is checked by, must not keep it
+  if (!*p) cudaGetLastError();
+  return *p != nullptr;
 }
 void dev_free(const lbcg_handle* h, void* p) {
   if (!p) return;
@@ -496,7 +500,6 @@ lbcg_status plan_run(lbcg_handle* h) {
   const size_t pb = p.tiles.size() * kRunFlagStride * sizeof(unsigned);
   // without memory for the plan the handle keeps one launch per kernel and step
   if (!dev_alloc(h, (void**)&h->d_run, host.size()) || !dev_alloc(h, (void**)&h->d_progress, pb)) {
-    cudaGetLastError();
     dev_free(h, h->d_run);
     h->d_run = nullptr;
     h->d_progress = nullptr;
@@ -1495,10 +1498,8 @@ lbcg_status adjoint_run(lbcg_handle* h, const lbcg_adjoint_spec* spec, lbcg_grad
   int rev_threads = 0;
   bool resident = !h->sweep && h->run_tiles > 0 && h->poll_limit == kPollLimit && !h->profiling;
   const size_t pb = size_t(h->run_tiles) * kRunFlagStride * sizeof(unsigned);
-  if (resident && (!B.get(&progress2, pb) || !B.get(&progress3, pb))) {
-    cudaGetLastError();
+  if (resident && (!B.get(&progress2, pb) || !B.get(&progress3, pb)))
     resident = false;   // without memory for the words: the launched stages
-  }
   if (resident) {
     CK(h, cudaMemsetAsync(progress2, 0, pb, h->stream));
     CK(h, cudaMemsetAsync(progress3, 0, pb, h->stream));

@@ -1,4 +1,4 @@
-"""lbcg_adjoint with an allocator that refuses one block."""
+"""lbcg_adjoint where device memory is refused."""
 import numpy as np
 import pytest
 
@@ -63,3 +63,25 @@ def test_adjoint_with_one_block_refused():
     finally:
         lbcg.lbcg_set_allocator()
     assert not held
+
+
+def test_refused_memory_is_not_the_next_launch_s_error():
+    # 10^10 states of checkpoint segments: cudaMalloc refuses them, the call reports it, and the handle
+    # and others step on
+    from paper_1707_00198_gb300 import lbcg
+    g, p = I.config_static_droplet()
+    L, other = lbcg.Lattice(g, p, "fp32"), lbcg.Lattice(g, p, "fp32")
+    w = np.ones((g.ny, g.nx))
+    for schedule in (lambda: L.set_tile(8), lambda: L.set_sweep()):
+        schedule()
+        with pytest.raises(lbcg.LBCGError) as ei:
+            L.adjoint(2, 10 ** 10, w)
+        assert ei.value.status == 8
+        L.step(1)
+        L.step(8)
+        with pytest.raises(lbcg.LBCGError):
+            L.adjoint(2, 10 ** 10, w)
+        other.step(1)
+        assert np.isfinite(L.populations()).all() and np.isfinite(other.populations()).all()
+    L.close()
+    other.close()
