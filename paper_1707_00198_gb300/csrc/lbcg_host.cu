@@ -1852,10 +1852,10 @@ lbcg_status lbcg_autotune(lbcg_handle* h, int32_t probe_steps, int32_t* schedule
       tile_ms = ms;
     }
   }
-  // the tile schedule's resident kernel, where it applies: it advances the state, which is
-  // saved and put back
+  // the tile schedule's resident kernel, where lbcg_step would take it: it advances the state, which
+  // is saved and put back
   if (e == cudaSuccess && s == LBCG_OK) s = plan_run(h);
-  if (e == cudaSuccess && s == LBCG_OK && h->run_tiles > 0) {
+  if (e == cudaSuccess && s == LBCG_OK && h->run_tiles > 0 && h->poll_limit == kPollLimit) {
     const size_t sb = lbcg_state_bytes(h);
     void* keep[2] = {nullptr, nullptr};
     if (dev_alloc(h, &keep[0], sb) && dev_alloc(h, &keep[1], sb)) {

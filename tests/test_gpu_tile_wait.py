@@ -71,3 +71,21 @@ def test_adjoint_reports_a_wait_that_ran_out_and_recovers(ckpt, fp32_reverse):
         assert np.array_equal(got[k], want[k]), k
     A.close()
     L.close()
+
+
+def test_autotune_leaves_out_a_kernel_that_steps_do_not_take():
+    # a changed lbcg_set_poll_limit keeps steps off the cooperative kernel: it is no candidate then (its
+    # waits, which would give up at once, are not reached)
+    from paper_1707_00198_gb300.lbcg import LBCGError
+    L = _lattice("fp32")
+    L.set_tile_poll_limit(0)
+    L.set_poll_limit(1 << 21)
+    s0 = L.populations()
+    L.autotune(4)
+    assert np.array_equal(L.populations(), s0)
+    L.set_poll_limit(-1)
+    L.autotune(4)               # as a candidate it does
+    with pytest.raises(LBCGError) as ei:
+        L.populations()
+    assert ei.value.status == LBCG_E_TIMEOUT
+    L.close()
