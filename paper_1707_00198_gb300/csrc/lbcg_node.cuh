@@ -121,7 +121,7 @@ __device__ __forceinline__ void grad_n_scheme_b(const T nxs[9], const T nys[9], 
 template <typename T>
 struct Collide {
   T ks, beta;                 // of the force: see csf_force
-  T hsum, hdiff, hR, hB;      // Eq. 18
+  T hlow, hdiff, hsign, hR, hB;   // Eq. 18, see viscous_rate
   T e1, e2, e3, e4, p1, p2, p3, p4, q1, q2, q3;
   __device__ __forceinline__ explicit Collide(const LatConst<T>& c) {
     beta = c.beta;
@@ -131,8 +131,10 @@ struct Collide {
     const T ce = fma_(T(-0.5), se, T(1)), cp = fma_(T(-0.5), sp, T(1)), cq = fma_(T(-0.5), sq, T(1));
     if constexpr (sizeof(T) == 8) {
       ks = rmul(c.sigma, T(1.0 / 24.0));
-      hsum = radd(c.h_inv_nuR, c.h_inv_nuB);
-      hdiff = rsub(c.h_inv_nuR, c.h_inv_nuB);
+      const bool red = c.h_inv_nuR >= c.h_inv_nuB;
+      hsign = red ? T(1) : T(-1);
+      hlow = rmul(T(2), red ? c.h_inv_nuB : c.h_inv_nuR);
+      hdiff = fabs(rsub(c.h_inv_nuR, c.h_inv_nuB));
       // relaxed e, eps and q moments with the weights of M^-1 (1/36, 1/36, 1/12) folded in:
       // e'/36 = e1 e + e2 rho u.u + e3 rho + e4 u.F, and so on
       constexpr T r36 = T(1) / T(36), r12 = T(1) / T(12);
@@ -155,7 +157,7 @@ struct Collide {
       p4 = cp;
       q1 = sq;
       q3 = cq;
-      hsum = hdiff = e2 = e3 = p2 = p3 = q2 = T(0);   // FP64 form only
+      hlow = hdiff = hsign = e2 = e3 = p2 = p3 = q2 = T(0);   // FP64 form only
     }
   }
 };
@@ -216,11 +218,14 @@ __device__ __forceinline__ void relax_rest(Moments<double>& m, double rho, const
   m.eps = fma_(c.p1, m.eps, rmul(c.p3, rho));
 }
 
-// s_v = 1/tau_v = 1/(3 nu + 1/2) (Eq. 5) with the harmonic viscosity of Eq. 18
+// s_v = 1/tau_v = 1/(3 nu + 1/2) (Eq. 5) with the harmonic viscosity of Eq. 18.  FP64: 1 / nu as the
+// smaller of the two plus their difference's share, two operations for four, exact in pure fluid on
+// that side (as the plain sum of the halves and rho^N times half the difference, pure fluid of the smaller 1 / nu was
+// off by the last bits of the larger).
 template <typename T>
 __device__ __forceinline__ T viscous_rate(T rn, const Collide<T>& c) {
   T inv_nu;
-  if constexpr (sizeof(T) == 8) inv_nu = fma_(rn, c.hdiff, c.hsum);
+  if constexpr (sizeof(T) == 8) inv_nu = fma_(fma_(c.hsign, rn, T(1)), c.hdiff, c.hlow);
   else inv_nu = fma_(radd(T(1), rn), c.hR, rmul(rsub(T(1), rn), c.hB));
   return rmul(inv_nu, rcp_(fma_(T(0.5), inv_nu, T(3))));
 }
