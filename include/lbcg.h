@@ -83,7 +83,8 @@ typedef struct {
                                   populations are f_{a,R} = w_a rho0 (1 + rhoN0)/2,
                                   f_{a,B} = w_a rho0 (1 - rhoN0)/2 at rest                 */
   const double* normal;        /* [2][ny*nx] analytic solid normal n_s pointing into the
-                                  solid (Sec. II.C.1.a, curved walls), or NULL to use the
+                                  solid (Sec. II.C.1.a, curved walls), used as given
+                                  (Eq. 34 is meant for unit length), or NULL to use the
                                   E8 estimate of Eq. 32-33                                 */
   const double* theta_node;    /* [ny*nx] contact angle per node in radians, or NULL to use
                                   lbcg_params.theta everywhere                             */

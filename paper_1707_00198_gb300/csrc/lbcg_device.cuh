@@ -89,7 +89,8 @@ struct LatDev {
   double nu_R, nu_B, sigma, beta, s_e, s_eps, s_q, rho0, u_in, rho_out, grad_eps;
   double h_inv_nuR, h_inv_nuB;  // 1/(2 nu_R), 1/(2 nu_B): the two weights of Eq. 18
   double in_y0, in_w;           // inlet profile: s = (y - in_y0) / in_w across the channel
-  int wetting, pad2_;           // 0: improved scheme (a); 1: scheme (b), Eq. 48; 2: surface energy
+  int wetting;                  // 0: improved scheme (a); 1: scheme (b), Eq. 48; 2: surface energy
+  int unit_normals;             // 1: every solid normal is of unit length, to rounding, or zero
   double cos_theta;             // cos(theta) of the surface-energy variant
   // the same constants rounded to FP32 on the host: a kernel that computes in FP32 otherwise
   // converts about ten doubles per thread, on an FP64 pipe of two lanes per SM

@@ -814,7 +814,13 @@ lbcg_status lbcg_create_batch(int32_t n, const lbcg_geometry* geoms, const lbcg_
   std::vector<uint8_t> mask_host((size_t)node_total, 0);
   for (int l = 0; l < n; ++l) {
     std::vector<uint8_t> fl, mk;
+    const size_t first = ofb.size();
     classify(&geoms[l], &prms[l], l, fl, mk, ofb);
+    // (a vector divided by its length is off by 6e-16 in its square at most)
+    ld[l].unit_normals = std::all_of(ofb.begin() + first, ofb.end(), [](const OfbEntry& e) {
+      const double n2 = e.nsx * e.nsx + e.nsy * e.nsy;
+      return std::fabs(n2 - 1.0) <= 1e-15 || n2 == 0.0;
+    });
     const LatHost& L = h->lats[l];
     for (int y = 0; y < L.ny; ++y) {
       memcpy(&h->flags_host[L.node_off + (size_t)y * L.pitch], &fl[(size_t)y * L.nx], L.nx);

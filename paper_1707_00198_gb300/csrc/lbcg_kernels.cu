@@ -48,7 +48,8 @@ template <typename T>
 __device__ __forceinline__ void wall_node(const LatDev& sL, const OfbEntry& e, const WallSten& q, const T* val,
                                           T* __restrict__ wall, long long node_total) {
   T cgx, cgy, nx, ny;
-  wall_normal<T>(T(sL.grad_eps), sL.wetting, T(e.nsx), T(e.nsy), T(e.cos_t), T(e.sin_t), q, val, cgx, cgy, nx, ny);
+  wall_normal<T>(T(sL.grad_eps), sL.wetting, sL.unit_normals, T(e.nsx), T(e.nsy), T(e.cos_t), T(e.sin_t), q, val, cgx,
+                 cgy, nx, ny);
   const long long k = sL.node_off + (long long)e.y * sL.pitch + e.x;
   wall[k] = cgx;
   wall[node_total + k] = cgy;

@@ -385,7 +385,7 @@ __device__ __forceinline__ bool near_tie(T d1, T d2) {
 // longest of the step.)  f1, f2: this component of the candidates; d_x, d_y: candidate r + 1.
 // All 32 lanes of the warp call it.
 template <typename T>
-__device__ __forceinline__ void wall_normal_pair(T eps, int wetting, T f1, T f2, T cx, T cy, const WallSten& q,
+__device__ __forceinline__ void wall_normal_pair(T eps, int wetting, bool unit, T f1, T f2, T cx, T cy, const WallSten& q,
                                                  const T* val, int r, T& cg, T& n) {
   auto v = [&](int a) { return rmul(wgt<T>(a), val[q.i[a - 1]]); };
   T g = rmul(wgt<T>(1), val[q.i[r]]);
@@ -413,7 +413,7 @@ __device__ __forceinline__ void wall_normal_pair(T eps, int wetting, T f1, T f2,
     const T a1 = rsub(cx, r ? eo : es), b1 = rsub(cy, r ? es : eo);
     const T d = radd(rmul(a1, a1), rmul(b1, b1)), od = other(d);
     bool one = r ? od <= d : d <= od;
-    const bool close = near_tie(d, od);
+    const bool close = !unit || near_tie(d, od);
     if (__any_sync(0xFFFFFFFFu, close)) {
       const T ge = rdiv(sum, T(1.0 / 3.0)), gge = rmul(ge, ge), mage = rsqrt_(radd(gge, other(gge)));
       const T ese = rdiv(ge, on ? mage : T(1)), eoe = other(ese);
@@ -425,6 +425,11 @@ __device__ __forceinline__ void wall_normal_pair(T eps, int wetting, T f1, T f2,
     if (on) {
       cg = rmul(mag, nf);
       n = nf;
+    }
+    if (!unit) {   // uniform over the block
+      sq = rmul(cg, cg);
+      const T m2 = rsqrt_(radd(sq, other(sq)));
+      if (on) n = m2 > eps ? rdiv(cg, m2) : T(0);
     }
   } else {
     const T mag = rsqrt_(radd(sq, other(sq)));
@@ -452,9 +457,11 @@ __device__ __forceinline__ void wall_normal_pair(T eps, int wetting, T f1, T f2,
 // in the oracle's order (directions 1..8, products w*phi then sign), so that a gradient exactly
 // along the wall's normal makes Eq. 35-36 an exact tie.  FP64 takes one reciprocal square root in
 // place of three square roots and seven divisions: it compares the squared distances (near a tie
-// the distances themselves) and takes n = n_f (30 operations against 78).
+// the distances themselves) and takes n = n_f (30 operations against 78).  That holds where the lattice's
+// solid normals are of unit length (unit: LatDev::unit_normals); given normals of another length take
+// the distances themselves and n = g_c / |g_c|.
 template <typename T>
-__device__ __forceinline__ void wall_normal(T eps, int wetting, T nsx, T nsy, T c, T s, const WallSten& q, const T* val,
+__device__ __forceinline__ void wall_normal(T eps, int wetting, bool unit, T nsx, T nsy, T c, T s, const WallSten& q, const T* val,
                                             T& cgx, T& cgy, T& nx, T& ny) {
   T gx = T(0), gy = T(0);
 #pragma unroll
@@ -485,7 +492,7 @@ __device__ __forceinline__ void wall_normal(T eps, int wetting, T nsx, T nsy, T 
     const T a1 = rsub(f1x, esx), b1 = rsub(f1y, esy), a2 = rsub(f2x, esx), b2 = rsub(f2y, esy);
     const T d1 = radd(rmul(a1, a1), rmul(b1, b1)), d2 = radd(rmul(a2, a2), rmul(b2, b2));
     bool one = d1 <= d2;
-    if (near_tie(d1, d2)) {
+    if (!unit || near_tie(d1, d2)) {
       const T gex = rdiv(sx, T(1.0 / 3.0)), gey = rdiv(sy, T(1.0 / 3.0));
       const T mage = rsqrt_(radd(rmul(gex, gex), rmul(gey, gey)));
       const T ex_ = rdiv(gex, mage), ey_ = rdiv(gey, mage);
@@ -496,6 +503,11 @@ __device__ __forceinline__ void wall_normal(T eps, int wetting, T nsx, T nsy, T 
     ny = one ? f1y : f2y;
     cgx = rmul(mag, nx);
     cgy = rmul(mag, ny);
+    if (!unit) {
+      const T m = rsqrt_(radd(rmul(cgx, cgx), rmul(cgy, cgy)));
+      nx = m > eps ? rdiv(cgx, m) : T(0);
+      ny = m > eps ? rdiv(cgy, m) : T(0);
+    }
     return;
   }
   const T cs2 = T(1.0 / 3.0);

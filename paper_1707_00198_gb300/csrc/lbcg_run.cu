@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(NT, run_blocks(sizeof(typename Store<S>::T))) 
       for (int j0 = w & ~31; j0 < 2 * tl.nw; j0 += kWallTeam) {   // two lanes per node, whole warps
         const int j = min((j0 + (w & 31)) >> 1, tl.nw - 1), r = w & 1;
         T g, n;
-        wall_normal_pair<T>(C.grad_eps, sL.wetting, sw[r * tl.nw + j], sw[(2 + r) * tl.nw + j],
+        wall_normal_pair<T>(C.grad_eps, sL.wetting, sL.unit_normals, sw[r * tl.nw + j], sw[(2 + r) * tl.nw + j],
                             sw[2 * r * tl.nw + j], sw[(2 * r + 1) * tl.nw + j], w_sten[j], swv, r, g, n);
         sw[(4 + r) * tl.nw + j] = g;   // (lanes past the end repeat the last node)
         sw[(6 + r) * tl.nw + j] = n;
