@@ -167,7 +167,7 @@ def kernel_source_digest() -> str:
     """Digest of the kernel sources' code: // comments and whitespace are left out, so that a
     comment edit does not invalidate counters taken from the same code."""
     h = hashlib.sha256()
-    for f in ("lbcg_kernels.cu", "lbcg_device.cuh", "lbcg_geom.h"):
+    for f in ("lbcg_kernels.cu", "lbcg_device.cuh", "lbcg_node.cuh", "lbcg_geom.h"):
         text = open(os.path.join(ROOT, "paper_1707_00198_gb300", "csrc", f), encoding="utf-8").read()
         code = "\n".join(" ".join(line.split("//", 1)[0].split()) for line in text.splitlines())
         h.update(code.encode())
