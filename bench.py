@@ -169,8 +169,8 @@ def kernel_source_digest() -> str:
     h = hashlib.sha256()
     for f in ("lbcg_kernels.cu", "lbcg_device.cuh", "lbcg_node.cuh", "lbcg_geom.h"):
         text = open(os.path.join(ROOT, "paper_1707_00198_gb300", "csrc", f), encoding="utf-8").read()
-        code = "\n".join(" ".join(line.split("//", 1)[0].split()) for line in text.splitlines())
-        h.update(code.encode())
+        lines = (" ".join(line.split("//", 1)[0].split()) for line in text.splitlines())
+        h.update("\n".join(line for line in lines if line).encode())
     return h.hexdigest()[:16]
 
 

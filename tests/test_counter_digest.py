@@ -1,4 +1,5 @@
-"""The digest that recorded counters carry sees every file whose code the sweeps are compiled from."""
+"""The digest that recorded counters carry sees every file whose code the sweeps are compiled from,
+and no comment."""
 import os
 import re
 import shutil
@@ -28,6 +29,8 @@ def test_an_edit_of_the_sweeps_code_changes_the_digest(tmp_path, monkeypatch):
     for f in sorted(files):
         path = tmp_path / CSRC / f
         text = path.read_text(encoding="utf-8")
+        path.write_text("// a comment\n\n" + text + "\n  // another\n", encoding="utf-8")
+        assert bench.kernel_source_digest() == want, f
         path.write_text(text + "\nint an_edit;\n", encoding="utf-8")
         assert bench.kernel_source_digest() != want, f
         path.write_text(text, encoding="utf-8")
