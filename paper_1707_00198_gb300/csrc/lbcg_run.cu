@@ -16,17 +16,17 @@
 // the two without a change of bits.
 //
 // What bounds it: on the smallest lattices the chain of one step (a flag's round trip through
-// L2, about 3300 cycles with the release of the stores before it, then the loads, the wall chain and the collision
-// of one pass); on the larger ones instruction issue; in FP64 the FP64 pipe.  Per step, launch per
-// kernel -> resident: 100 x 50 FP64 26.5 -> 12.6 us, 1200 x 80 FP64 72 -> 35.5, FP32 10.5 -> 5.3,
-// 2000 x 102 FP32 17.3 -> 9.4, FP16 18.6 -> 9.3, 8 x 630 x 60 FP32 with Poiseuille inlets 36 -> 12.8
+// L2, about 3300 cycles with the release of the stores before it, then the loads, the wall chain and
+// the collision of one pass); on the larger ones instruction issue; in FP64 the FP64 pipe.  Per step,
+// launch per kernel -> resident: 100 x 50 FP64 26.5 -> 12.6 us, 1200 x 80 FP64 72 -> 35.5, FP32 10.5 ->
+// 5.3, 2000 x 102 FP32 17.3 -> 9.4, FP16 18.6 -> 9.3, 8 x 630 x 60 FP32 with Poiseuille inlets 36 -> 12.8
 // (18.4 with the inlet profile evaluated, in FP64, at every read of an edge node).  FP32 arithmetic:
 // two blocks of 256 threads per SM, whose waits overlap each other's work, against one of 512:
 // 2000 x 102 FP32 9.4 -> 9.1, FP16 9.3 -> 8.7, 8 x 630 x 60 12.8 -> 11.8; with the push offsets of
 // bulk nodes apart from those of wall nodes 8.7, 8.5 and 11.3.  FP64 with one reciprocal square root
-// per node in the wall chain (lbcg_node.cuh): 100 x 50 12.6 -> 10.5 us, 1200 x 80 35.5 -> 35.2,
-// 2000 x 102 123 -> 111 (9.9, 34.6 and 111 with the divisions of rho^N and of Eq. 29 also reciprocals, which
-// decides near ties of Eq. 36 otherwise than the equations' own operations).
+// per node in the wall chain (lbcg_node.cuh): 100 x 50 12.6 -> 10.6 us, 1200 x 80 35.5 -> 35.4,
+// 2000 x 102 123 -> 111 (9.9, 34.6 and 111 with the divisions of rho^N and of Eq. 29 also reciprocals,
+// which decides near ties of Eq. 36 otherwise than the equations' own operations).
 #include "lbcg_internal.h"
 #include "lbcg_node.cuh"
 #include "lbcg_wait.cuh"
@@ -107,6 +107,9 @@ __global__ void __launch_bounds__(NT, run_blocks(sizeof(typename Store<S>::T))) 
   const LatConst<T> C = sL.consts<T>();
   const Collide<T> K(C);
   const T eps2 = rmul(C.grad_eps, C.grad_eps);
+  // (in registers: read from shared memory in every step, 2000 x 102 FP16 8.36 us per step, for 8.33)
+  const int wetting = sL.wetting;
+  const bool unit = sL.unit_normals;
   const uint8_t* __restrict__ fl = A.flags + sL.node_off;
   const uint8_t* __restrict__ nbm = A.nbmask + sL.node_off;
   const long long pop_off = sL.pop_off, pop_n = 18 * sL.plane;
@@ -271,12 +274,12 @@ __global__ void __launch_bounds__(NT, run_blocks(sizeof(typename Store<S>::T))) 
     } else {
       const int w = t - team;
       for (int j = w; j < tl.nv; j += kWallTeam)
-        swv[tl.nband + j] = sL.wetting == 2 ? C.cos_theta : virtual_value<T>(v_sten[j], swv, sden[j]);
+        swv[tl.nband + j] = wetting == 2 ? C.cos_theta : virtual_value<T>(v_sten[j], swv, sden[j]);
       bar_sync(1, kWallTeam);
       for (int j0 = w & ~31; j0 < 2 * tl.nw; j0 += kWallTeam) {   // two lanes per node, whole warps
         const int j = min((j0 + (w & 31)) >> 1, tl.nw - 1), r = w & 1;
         T g, n;
-        wall_normal_pair<T>(C.grad_eps, sL.wetting, sL.unit_normals, sw[r * tl.nw + j], sw[(2 + r) * tl.nw + j],
+        wall_normal_pair<T>(C.grad_eps, wetting, unit, sw[r * tl.nw + j], sw[(2 + r) * tl.nw + j],
                             sw[2 * r * tl.nw + j], sw[(2 * r + 1) * tl.nw + j], w_sten[j], swv, r, g, n);
         sw[(4 + r) * tl.nw + j] = g;   // (lanes past the end repeat the last node)
         sw[(6 + r) * tl.nw + j] = n;
@@ -328,7 +331,7 @@ __global__ void __launch_bounds__(NT, run_blocks(sizeof(typename Store<S>::T))) 
       T dxx, dxy, dyx, dyy;
       grad_n<T>(snx + o1, sny + o1, PW, dxx, dyx, dxy, dyy);
       const unsigned mask = e & 0xFFu;
-      if (sL.wetting == 1 && (e & kOwnOfb)) {
+      if (wetting == 1 && (e & kOwnOfb)) {
         T nxs[9], nys[9];
 #pragma unroll
         for (int a = 0; a < 9; ++a) {
