@@ -246,8 +246,8 @@ lbcg_status lbcg_set_tile(lbcg_handle* h, int32_t ty);
  * The cooperative kernels (of long calls of lbcg_step, and of lbcg_adjoint) have the other
  * device-side wait, of a tile for the tiles around it, with a bound of its own,
  * lbcg_set_tile_poll_limit (the same default and the same meaning of polls), and reported the same
- * way, by lbcg_adjoint itself where it happens there.  A handle whose lbcg_set_poll_limit was changed launches
- * each kernel of its steps instead. */
+ * way, by lbcg_adjoint itself where it happens there.  A handle whose lbcg_set_poll_limit was changed
+ * launches each kernel of its steps instead. */
 lbcg_status lbcg_set_poll_limit(lbcg_handle* h, int32_t polls);
 lbcg_status lbcg_set_tile_poll_limit(lbcg_handle* h, int32_t polls);
 
@@ -293,8 +293,8 @@ lbcg_status lbcg_adjoint(lbcg_handle* h, const lbcg_adjoint_spec* spec, lbcg_gra
  * 64 and 80 rows; tiles 4, 8, 16) as lbcg_step runs it, a captured graph of `probe_steps`
  * steps (with a batch's parallel branches) that rewrite the same next state from the current
  * one without advancing it, and the tiles as the cooperative kernel of long calls (the state is
- * saved and put back; not with a changed lbcg_set_poll_limit, which keeps steps off it), keeps the fastest and writes it to *schedule (0 = sweep, else the tile height;
- * schedule may be NULL).  It synchronises the handle's stream.  The candidates
+ * saved and put back; not with a changed lbcg_set_poll_limit, which keeps steps off it), keeps the
+ * fastest and writes it to *schedule (0 = sweep, else the tile height; schedule may be NULL).  It synchronises the handle's stream.  The candidates
  * give the same result up to rounding order (FP32: a few ulp per step; FP64 within 1e-13).
  * lbcg_schedule reports the current choice with the same encoding, lbcg_sweep_rows the
  * sweep's rows per strip segment (0: the automatic height; -1 for a NULL handle). */

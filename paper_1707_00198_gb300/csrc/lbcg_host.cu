@@ -80,7 +80,7 @@ struct lbcg_handle {
   uint8_t* d_flags = nullptr;
   uint8_t* d_nbmask = nullptr;
   int scheme_b = 0;        // some lattice uses wetting scheme (b)
-  int* d_err = nullptr;    // device error word (a sweep block's bounded wait ran out)
+  int* d_err = nullptr;    // device error word (a bounded wait of a step or reverse kernel ran out)
   int poll_limit = kPollLimit;   // polls of a sweep block's wait for a staged row (about a second)
   int run_polls = kPollLimit;    // and of a resident kernel's wait for the tiles around one
   uint32_t* d_sr_epoch = nullptr;     // 16-bit storage: graph replays so far (stochastic-rounding keys)
@@ -109,8 +109,8 @@ struct lbcg_handle {
     double v[kObsOut];
   };
   Small* h_small = nullptr;
-  // the resident kernel of the tile schedule (calls of more than kGraphSteps steps): its plan
-  // on the device, or run_tiles = 0 where the lattices do not fit
+  // the resident kernel of the tile schedule (see runs_resident): its plan on the device, or
+  // run_tiles = 0 where the lattices do not fit
   bool run_planned = false;
   int run_tiles = 0;
   size_t run_smem = 0;
@@ -456,11 +456,11 @@ lbcg_status plan_run(lbcg_handle* h) {
   }
   // (a fluid node takes at least its 12 values and 8 bytes of tables)
   if (fluid * (long long)(12 * cs + 8) > (long long)sms * blocks * (long long)budget) return LBCG_OK;
-  // Small lattices take blocks that leave room on their SMs for those of other handles: a cooperative grid
-  // starts only once all its blocks have room, so that grids of large blocks run one after another.
-  // FP32: one tile per SM, where 128 threads take each stage of it in one pass, is as fast as two half as
-  // large (100 x 50: 3.30 us per step either way), and eight handles at once on streams of their own take 0.92 us per
-  // step of each, for 1.75.  16-bit storage keeps two (3.27 us, one 3.37).
+  // Small lattices take blocks that leave room on their SMs for those of other handles: a cooperative
+  // grid starts only once all its blocks have room, so that grids of large blocks run one after another.
+  // FP32: one tile per SM, where 128 threads take each stage of it in one pass, is as fast as two half
+  // as large (100 x 50: 3.30 us per step either way), and eight handles at once on streams of their own
+  // take 0.92 us per step of each, for 1.75.  16-bit storage keeps two (3.27 us, one 3.37).
   RunPlan p;
   const bool one = h->prec == LBCG_FP32 && fluid <= (long long)kRunSmallThreads / 2 * sms &&
                    build_run_plan(views, flags, h->ofb_host, sms, budget, cs, p) && run_one_pass(p);
@@ -469,10 +469,12 @@ lbcg_status plan_run(lbcg_handle* h) {
     h->run_nodes = std::max(h->run_nodes, t.tx * t.ty);
     h->run_slots = std::max(h->run_slots, (t.tx + 4) * (t.ty + 4));
   }
-  // Blocks of 128 threads where the tiles are that small.  FP32: they also leave registers for a kernel on
-  // another stream (the adjoint's reverse sweep beside the recompute of a segment).  FP64: where
-  // each stage is one pass of them (100 x 50: 10.5 us per step either way; eight handles at once 6.0 us
-  // per step of each, for 10.6; with two passes 1.1 to 1.2 times the time of 256 threads).
+  // Blocks of 128 threads where the tiles are that small.  FP32: they also leave registers for a kernel
+  // on another stream, the adjoint's reverse sweep beside the recompute of a segment (400 x 42: 20 us per
+  // step of the gradient, for 23 with 256 threads, although the steps alone take 4.27 us, for 3.99; 100 x 50
+  // 3.35 and 3.38, in FP16 3.42 and 3.55).  FP64: where each stage is one pass of them (100 x 50: 10.6 us
+  // per step either way; eight handles at once 6.0 us per step of each, for 10.6; with two passes 1.1
+  // to 1.2 times the time of 256 threads).
   h->run_threads = (cs == 4 ? h->run_nodes <= 64 : run_one_pass(p)) ? kRunSmallThreads : 256;
   int per_sm = 0;
   CK(h, prepare_run(h->prec, h->run_threads, p.smem, &per_sm));
@@ -539,7 +541,8 @@ lbcg_status plan_run(lbcg_handle* h) {
 // Profiled handles (events around each kernel), handles whose poll limit was changed and
 // streams that are being captured keep the launch-per-step schedule.
 bool runs_resident(const lbcg_handle* h, int64_t nsteps) {
-  if (h->sweep || h->run_tiles == 0 || nsteps < kRunMinSteps || nsteps == kGraphSteps || h->profiling || h->poll_limit != kPollLimit) return false;
+  if (h->sweep || h->run_tiles == 0 || h->profiling || h->poll_limit != kPollLimit) return false;
+  if (nsteps < kRunMinSteps || nsteps == kGraphSteps) return false;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   return cudaStreamIsCapturing(h->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
 }
@@ -577,10 +580,10 @@ lbcg_status ensure_macro(lbcg_handle* h) {
   return LBCG_OK;
 }
 
-// After a synchronisation: a sweep block gave up waiting for a staged row (or a block of the
-// resident kernel for a tile next to it), so the state of the steps since the last check is
-// unreliable (that block stopped without writing the rest).  The word is cleared once reported: the handle stays usable, and a state set
-// or uploaded afterwards steps correctly again.
+// After a synchronisation: a sweep block gave up waiting for a staged row (or a block of a resident
+// kernel for a tile next to it), so the state of the steps since the last check is unreliable (that
+// block stopped without writing the rest).  The word is cleared once reported: the handle stays
+// usable, and a state set or uploaded afterwards steps correctly again.
 lbcg_status report_device_error(lbcg_handle* h, int e) {
   if (e) {
     // (on the handle's stream: before what is launched next)

@@ -220,8 +220,9 @@ __device__ __forceinline__ void relax_rest(Moments<double>& m, double rho, const
 
 // s_v = 1/tau_v = 1/(3 nu + 1/2) (Eq. 5) with the harmonic viscosity of Eq. 18.  FP64: 1 / nu as the
 // smaller of the two plus their difference's share, two operations for four, exact in pure fluid on
-// that side (as the plain sum of the halves and rho^N times half the difference, pure fluid of the smaller 1 / nu was
-// off by the last bits of the larger).
+// that side (as the sum of the halves plus rho^N times half their difference, one operation, pure
+// fluid of the smaller 1 / nu was off by the last bits of the larger; 100 x 50 10.57 us per step, now
+// 10.64, 1200 x 80 35.2, now 35.4).
 template <typename T>
 __device__ __forceinline__ T viscous_rate(T rn, const Collide<T>& c) {
   T inv_nu;

@@ -8,12 +8,13 @@ namespace lbcg {
 
 size_t run_smem_bytes(const RunTile& t, size_t cs) {
   auto up = [](size_t b) { return (b + 15) & ~size_t(15); };
-  const size_t nr = size_t(t.tx + 4) * (t.ty + 4) + t.ne, np = size_t(t.tx + 2) * (t.ty + 2), no = size_t(t.tx) * t.ty;
-  return up(nr * cs) + up((size_t(t.nband) + t.nv) * cs) + 4 * up(np * cs) + up(12 * no * cs) + up(8 * size_t(t.nw) * cs) +
-         up((size_t(t.nv) + t.nvn) * cs) +
-         up(nr * 4) * 2 + up(nr * 2) + up((size_t(t.ty) + 8) * cs) + up(np * 2) + up(no * 4) + up((size_t(t.tx) + 2) * 4) + up((size_t(t.ty) + 2) * 4) +
-         up(t.nw * sizeof(WallSten)) + up(t.nv * sizeof(WallSten)) + up(t.nvn * sizeof(RunVirtN)) +
-         up(size_t(t.ncopy) * 4);
+  const size_t nr = size_t(t.tx + 4) * (t.ty + 4) + t.ne, np = size_t(t.tx + 2) * (t.ty + 2);
+  const size_t no = size_t(t.tx) * t.ty;
+  return up(nr * cs) + up((size_t(t.nband) + t.nv) * cs) + 4 * up(np * cs) + up(12 * no * cs) +
+         up(8 * size_t(t.nw) * cs) + up((size_t(t.nv) + t.nvn) * cs) + up(nr * 4) * 2 + up(nr * 2) +
+         up((size_t(t.ty) + 8) * cs) + up(np * 2) + up(no * 4) + up((size_t(t.tx) + 2) * 4) +
+         up((size_t(t.ty) + 2) * 4) + up(t.nw * sizeof(WallSten)) + up(t.nv * sizeof(WallSten)) +
+         up(t.nvn * sizeof(RunVirtN)) + up(size_t(t.ncopy) * 4);
 }
 
 bool run_one_pass(const RunPlan& plan) {

@@ -53,7 +53,7 @@ struct RunPlan {
   size_t smem = 0;                // dynamic shared memory of the largest tile
 };
 
-// Blocks, i.e. tiles, per SM for `cs` bytes per value of the compute type.  FP32 arithmetic: two, so
+// Blocks, i.e. tiles, per SM, at most, for `cs` bytes per value of the compute type.  FP32 arithmetic: two, so
 // that one works while the other waits for its neighbours.  FP64: one, since the FP64 pipe is
 // the bound and a tile half as large recomputes more of its halo.
 LBCG_HD constexpr int run_blocks(size_t cs) { return cs == 4 ? 2 : 1; }
